@@ -1303,8 +1303,8 @@ int batch_plan_merge(ej_batch *b) {
     }
     for (int i : pq) {
         const BatchJoin &j = b->joins[(size_t)i];
-        own += (double)j.ncand * pq_words(j.p.K);
-        wide += (double)j.ncand * W1;
+        own += (double)j.ncand * (pq_words(j.p.K) + 1);   // a column costs about one word more than its window
+        wide += (double)j.ncand * (W1 + 1);
     }
     if (mode == 0 && wide > 1.5 * own) return EJ_OK;
     const int threads = pq_threads_for(W1, b->joins[0].p.alphabet_size);
@@ -1370,8 +1370,7 @@ int batch_merged_verify(ej_batch *b, cudaStream_t s) {
     }
     CK(launch_verify_pq(b->mW1, b->mthreads, ctx->sched.slots_per_warp ? ctx->sched.slots_per_warp : 16,
                         ctx->sched.warps_per_subpartition, pl.packed, pl.pofs,
-                        pl.B, pl.lens, pl.st.n, b->joins[0].p.alphabet_size, nullptr, (int64_t)total_cap, b->mK, vo, s,
-                        b->munion));   // the union launch runs only while its pairs are few
+                        pl.B, pl.lens, pl.st.n, b->joins[0].p.alphabet_size, nullptr, (int64_t)total_cap, b->mK, vo, s));
     return EJ_OK;
 }
 

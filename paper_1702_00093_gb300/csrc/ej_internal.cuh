@@ -451,24 +451,23 @@ cudaError_t launch_verify(VerifyConfig c, const uint4 *packed, const uint64_t *p
                           const uint64_t *pairs, int64_t np, int32_t K, int64_t max_len,
                           VerifyOut vo, cudaStream_t s);
 
-// Persistent verifier (two lanes per pair, W1 = 2..12 words per lane, pairs
-// pulled from vo.queue). spw_force > 0 fixes the pair slots per warp (1..16);
-// wps > 0 caps the working warps at wps per SM sub-partition (slots refill).
-// Words per lane the persistent verifier needs for threshold K: its band has at
-// most K + 1 diagonals (the length difference narrows Ukkonen's 2K + 1), so
-// 1 + ceil(K / 64), at least 2.
+// Persistent verifier (two lanes per pair, a window of W 32-bit words per lane,
+// pairs pulled from vo.queue). spw_force > 0 fixes the pair slots per warp
+// (1..16); wps > 0 caps the working warps at wps per SM sub-partition (slots
+// refill).
+// Words per lane the persistent verifier uses for threshold K: its band has at
+// most K + 1 diagonals (the length difference narrows Ukkonen's 2K + 1), one bit
+// each. Every count up to 12 is compiled, then 16 and 24 (K <= 767).
+constexpr int PQ_MAX_WORDS = 24;
 inline int pq_words(int32_t K) {
-    const int w = 1 + (K + 63) / 64;
-    return w < 2 ? 2 : w;
+    const int w = (K + 32) / 32;
+    return w <= 12 ? w : w <= 16 ? 16 : w <= PQ_MAX_WORDS ? PQ_MAX_WORDS : w;
 }
-size_t pq_smem_bytes(int W1, uint32_t alpha, int threads);
-int pq_threads_for(int W1, uint32_t alpha);   // 0 if no block size fits
-// lean: the variant for launches set by their longest pairs (few pairs per
-// slot): chunks in which every running pair has all its columns skip the
-// per-column guard (a second copy of the column loop)
-cudaError_t launch_verify_pq(int W1, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
+size_t pq_smem_bytes(int W, uint32_t alpha, int threads);
+int pq_threads_for(int W, uint32_t alpha);   // 0 if no block size fits
+cudaError_t launch_verify_pq(int W, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
                              const int32_t *lens, int64_t n, uint32_t alpha, const uint64_t *pairs, int64_t np,
-                             int32_t K, VerifyOut vo, cudaStream_t s, bool lean = false);
+                             int32_t K, VerifyOut vo, cudaStream_t s);
 // Shared-string verifier (W1 = 2..12): the pairs of tasks[0 .. *ntasks_dev)
 // (at most ntasks_cap), each task up to 16 pairs sharing their longer string.
 cudaError_t launch_verify_sx(int W1, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,

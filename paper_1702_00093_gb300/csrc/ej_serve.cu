@@ -310,9 +310,9 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
         vo.thr = qK;
         vo.pairs_off_dev = bins + nc + c;
         const int W1 = pq_words(kband[c]);   // the persistent verifier's narrower band
-        const int threads = W1 <= 12 ? pq_threads_for(W1, alpha) : 0;
+        const int threads = pq_threads_for(W1, alpha);
         if (threads > 0) {
-            SV(launch_verify_pq(W1, threads, 16, 1, P<uint4>(sl.qpacked), P<uint64_t>(sl.qpofs), x.set.B,
+            SV(launch_verify_pq(W1, threads, 16, 0, P<uint4>(sl.qpacked), P<uint64_t>(sl.qpofs), x.set.B,
                                 P<int32_t>(sl.qlens), Q, alpha, P<uint64_t>(sl.cand), (int64_t)cap, kband[c], vo, s));
         } else {
             const VerifyConfig vc = verify_pick(kband[c], alpha, max_len);

@@ -4,7 +4,7 @@
 // takes the next one instead of idling until the slowest pair of its warp ends.
 //
 // Per pair, two lanes: the forward half computes D(., n1) for n1 = n/2 over a
-// block-aligned window of W1 64-row words, the backward half runs the same
+// diagonal window (ej_diag.cuh), the backward half runs the same
 // recurrence on the reversed strings for the remaining n - n1 columns, and
 // ED(x, y) = min_i D(i, n1) + ED(x[i:], y[n1:]) joins them (the argument and the
 // boundary conditions are the ones of the block-aligned two-lane verifier).
@@ -15,26 +15,34 @@
 // stays on the diagonals i - j in [-K_lo, K_hi], K_lo = floor((K - d) / 2),
 // K_hi = floor((K + d) / 2): at most K + 1 diagonals, where Ukkonen's band has
 // 2K + 1 (the same argument as his cutoff). Both halves use it (reversing both
-// strings keeps d). The window of W1 words covers it when W1 >= 1 + K/64
-// rounded up, moving down one word before the columns K_lo + 1 + 64t, t >= 1.
+// strings keeps d). The window is diagonal (ej_diag.cuh): W = ceil((K + 1) / 32)
+// 32-bit words hold exactly those diagonals.
 //
-// Scheduling. A warp advances its 16 pair slots in chunks of 64 columns. A slot
-// starts a new pair at a chunk boundary, its column 1 at chunk position s0 =
-// (smove - K_lo) mod 64 (the positions before it idle), so that every window
-// move of every pair falls on the same chunk position smove and runs once per
-// chunk for the whole warp. A finished slot waits at most one chunk. The number
-// of working warps is capped (by default one per SM sub-partition), so that a
-// batch larger than the slots keeps every slot busy until the queue runs dry.
+// Scheduling. A warp advances its 16 pair slots in chunks of 32 columns, one
+// match-mask word of the window entering per chunk. Both halves of a pair are
+// padded in front with a common prefix (which changes no distance) to the same
+// multiple of 32 columns, N1 = 32 ceil((n - floor(n/2)) / 32): every slot starts
+// and ends at a chunk boundary, both lanes of a slot together, and the column
+// loop has no test (a lane without a pair advances values that nothing reads; its
+// reads stay inside its own ring and the packed strings). The number of working
+// warps is capped (by default one per SM sub-partition), so that a batch larger
+// than the slots keeps every slot busy until the queue runs dry.
 //
-// Early exit. Once per chunk, at the chunk position of the window moves, each
-// half that is still running computes the minimum value m_h of its window
-// (including the row above it). A path of cost <= K crosses both halves'
+// Early exit. Every other chunk each half computes the minimum value m_h of its
+// window (including the top cell). A path of cost <= K crosses both halves'
 // current columns inside their bands, where the values are exact, so
 // m_fwd + m_bwd > K proves ED > K; both lanes of the pair stop.
+//
+// What bounds it: 32-bit integer instructions, 10 W + about 8 per column. With
+// many pairs (5.4M candidates of 20000 reads of 5000 bases at K = 250) the launch
+// takes 21.7 ms at three warps per sub-partition (23.8 at two, 33.2 at one),
+// against 28.2 ms for the block-aligned window with a test per column that this
+// form replaces; with few (about 13000, K = 250) it is set by the columns of its
+// longest pairs on one warp per sub-partition, 0.38 against 0.50 ms, and 0.25
+// against 0.49 ms at K = 150 (5 words against 8).
 #include <climits>
-#include <type_traits>
 
-#include "ej_bitpar.cuh"
+#include "ej_diag.cuh"
 
 namespace ej {
 
@@ -82,7 +90,56 @@ __device__ __forceinline__ uint64_t sym_reverse(uint64_t u) {
     return ((r >> 1) & 0x5555555555555555ull) | ((r & 0x5555555555555555ull) << 1);
 }
 
-template <int W1, int B, int TPB, bool LEAN>
+// Match-mask word of a pair's padded x (or reversed x) from symbol q on (bit t:
+// symbol q + t; symbols -pad .. -1 are the padding, code 0; none outside
+// [-pad, m)) for every symbol c < alpha, into ring entries c * R2 + slot and,
+// R entries further, its twin.
+template <int B, int R>
+__device__ __forceinline__ void pq_build(uint32_t *ring, int T_, int slot, const uint64_t *__restrict__ x64, int32_t m,
+                                         int64_t q, int32_t pad, bool rev, uint32_t alpha) {
+    constexpr int R2 = 2 * R;
+    const int t_lo = (int)max((int64_t)0, -(q + pad)), t_hi = (int)min((int64_t)32, m - q);
+    uint32_t valid = 0u;
+    if (t_hi > t_lo) valid = (t_hi >= 32 ? ~0u : (1u << t_hi) - 1u) & ~((1u << t_lo) - 1u);
+    const int64_t xwords = 2 * chunks_for(m, B);
+    if (B == 2) {
+        const uint64_t v = sym_join(sym_fetch<2>(x64, xwords, rev ? m - 32 - q : q));
+        const uint32_t w0 = (uint32_t)v, w1 = (uint32_t)(v >> 32);
+        uint32_t lo = compress_even(w0) | (compress_even(w1) << 16);
+        uint32_t hi = compress_even(w0 >> 1) | (compress_even(w1 >> 1) << 16);
+        if (rev) {
+            lo = __brev(lo);
+            hi = __brev(hi);
+        }
+        for (uint32_t c = 0; c < alpha; c++) {
+            const uint32_t e = ((c & 1u) ? lo : ~lo) & ((c & 2u) ? hi : ~hi) & valid;
+            ring[(size_t)(c * R2 + slot) * T_] = e;
+            ring[(size_t)(c * R2 + slot + R) * T_] = e;
+        }
+    } else {
+        for (uint32_t c = 0; c < alpha; c++) ring[(size_t)(c * R2 + slot) * T_] = 0u;
+        if (valid) {
+            // every symbol sets its bit with a shared-memory OR that returns
+            // nothing, so consecutive symbols (which may hit the same word) do
+            // not wait on one another
+#pragma unroll
+            for (int g = 0; g < 4; g++) {
+                uint64_t v = sym_join(sym_fetch<8>(x64, xwords, rev ? m - 8 - q - 8 * g : q + 8 * g));
+                if (rev) v = sym_reverse<8>(v);
+#pragma unroll
+                for (int t = 8 * g; t < 8 * g + 8; t++) {
+                    const uint32_t c = (uint32_t)v & 0xFFu;
+                    v >>= 8;
+                    if (t >= t_lo && t < t_hi) atomicOr(ring + (size_t)(c * R2 + slot) * T_, 1u << t);
+                }
+            }
+        }
+        for (uint32_t c = 0; c < alpha; c++)
+            ring[(size_t)(c * R2 + slot + R) * T_] = ring[(size_t)(c * R2 + slot) * T_];
+    }
+}
+
+template <int W, int B, int TPB>
 __global__ void __launch_bounds__(TPB, 1)
 verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ pofs,
                  const int32_t *__restrict__ lens, int64_t n_str, uint32_t alpha,
@@ -140,39 +197,30 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             if (idx < sg_.app_cap) sg_.app[idx] = sg_.pairs[q];
         }
     };
-    constexpr int R = W1 + 1;
+    constexpr int R = W + 1;                 // words of the window at any shift
     constexpr int R2 = 2 * R;                // ring slots per symbol: every word is kept twice,
                                              // at slot k mod R and k mod R + R, so that the
-                                             // window's W1 words sit at consecutive slots
+                                             // window's words sit at consecutive slots
     constexpr int SPW = 64 / B;              // symbols per 64-bit word
-    constexpr uint64_t CMASK = (1ull << B) - 1ull;
-    extern __shared__ uint64_t smem[];
-    __shared__ int8_t s_nsum[256];
-    __shared__ int8_t s_nmin[256];
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
-        const uint32_t P = t & 15u, M = t >> 4;
-        int run = 0, mn = 1 << 20;
-        for (int k = 0; k < 4; k++) {
-            run += (int)((P >> k) & 1u) - (int)((M >> k) & 1u);
-            mn = run < mn ? run : mn;
-        }
-        s_nsum[t] = (int8_t)run;
-        s_nmin[t] = (int8_t)mn;
-    }
+    constexpr uint32_t CMASK = (1u << B) - 1u;
+    extern __shared__ uint32_t pq_smem[];
+    __shared__ uint32_t s_tab[256];
+    diag_fill_table(s_tab);
     __syncthreads();
     if (segs) np = s_cum[nseg];
     constexpr int T_ = TPB;                   // slot stride of the per-thread ring
-    uint64_t *ring = smem + threadIdx.x;      // (c*R2 + slot)*T_, reused as a dump area
+    uint32_t *ring = pq_smem + threadIdx.x;   // (c*R2 + slot)*T_, reused as a dump area
     const int lane = threadIdx.x & 31;
     const bool rev = lane & 1;
     const int slot = lane >> 1;
-    const int32_t smove = K & 63;             // chunk position of every window move
-    const uint32_t cmax = alpha - 1u;
 
-    // Slots per warp and working warps. The working warps are chosen per SM
+    // Slots per warp and working warps. The working blocks are chosen per SM
     // (the first ones to take a ticket on their SM), so that they are spread
-    // evenly over the SMs whatever order the blocks were placed in; at most
-    // 4*wps per SM (wps per sub-partition), fewer when the batch is small.
+    // evenly over the SMs whatever order the blocks were placed in. A block of
+    // four warps has one on each sub-partition and takes one ticket: tickets per
+    // warp let the first warps of two blocks that start together land on the
+    // same sub-partitions (0.61 instead of 0.38 ms for the headline batch's
+    // launch). One-warp blocks: at most 4*wps per SM, fewer when the pairs are few.
     const int64_t spw = spw_force > 0 ? (spw_force > 16 ? 16 : spw_force) : 16;
     const int64_t warps_needed = (np + spw - 1) / spw;
     int64_t per_sm = (warps_needed + nsm - 1) / (nsm > 0 ? nsm : 1);
@@ -186,10 +234,11 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         wps = per_slot >= 32 ? 4 : per_slot >= 8 ? 2 : 1;
     }
     if (per_sm > 4ll * wps) per_sm = 4ll * wps;
-    unsigned ticket = 0;
-    if (lane == 0) ticket = atomicAdd(&vo.sm_tickets[sm_id() & (SM_TICKETS - 1)], 1u);
-    ticket = __shfl_sync(FULL, ticket, 0);
-    bool exhausted = (slot >= spw) || ((int64_t)ticket >= per_sm);
+    constexpr int BW = TPB / 32;
+    __shared__ unsigned s_ticket;
+    if (threadIdx.x == 0) s_ticket = atomicAdd(&vo.sm_tickets[sm_id() & (SM_TICKETS - 1)], 1u);
+    __syncthreads();
+    bool exhausted = (slot >= spw) || ((int64_t)s_ticket >= (per_sm + BW - 1) / BW);
     if (__all_sync(FULL, exhausted)) return;
     // merged launch: the warp's work counters per join, in shared memory (added
     // to the joins' global counters once, when the warp ends)
@@ -200,33 +249,30 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
 
     unsigned long long loc_cells = 0, loc_cols = 0;
     bool have = false, rejected = false;
-    int64_t p = 0, k0 = 0;
-    const uint4 *xc = packed;
-    const uint64_t *y64 = reinterpret_cast<const uint64_t *>(packed);
+    int64_t p = 0;
+    const uint64_t *x64 = reinterpret_cast<const uint64_t *>(packed), *y64 = x64;
     int64_t ywords = 0;
-    int32_t m = 0, n = 0, ncols = 0, Tacc = 0, jbase = 1, next_move = 0, rej_col = 0;
+    int32_t m = 0, n = 0, klo = 0, T = 0;
+    int32_t ncols = 0;       // padded columns of either half (a multiple of 32)
+    int32_t pad = 0;         // padding columns of this lane's half
+    int32_t j0 = 0;          // columns done
     int32_t wpair = 1;       // words of the pair's band, ceil((K_lo + K_hi + 1) / 64) (work counter)
-    // the raw word of y's (or reversed y's) symbols from symbol index sidx on
-    auto sym_word = [&](int64_t sidx) -> SymRaw {
-        return sym_fetch<B>(y64, ywords, rev ? (int64_t)n - SPW - sidx : sidx);
+    // the raw word of padded y's (or reversed y's) symbols from column sidx + 1 on
+    auto sym_word = [&](int32_t sidx) -> SymRaw {
+        const int64_t q = (int64_t)sidx - pad;
+        return sym_fetch<B>(y64, ywords, rev ? (int64_t)n - SPW - q : q);
     };
     SymRaw snext{0ull, 0ull, 0u};   // the next word of the stream, already requested
     int32_t kp = K;          // the pair's threshold (<= K, the band)
     int sg = 0;              // the pair's join (merged launch; of the union: the largest K's)
     uint32_t umk = 0;        // union pair: the mask of the joins that list it
-    int32_t budget = 0;      // chunks this pair may still take (ncols/64 + 2 suffice)
-    int64_t iters = 0;       // loop passes of this warp (bounded by max_iters)
-    const int64_t max_iters = vo.max_passes > 0 ? vo.max_passes : kMaxIters;
+    int64_t iters = 0;       // chunks of this warp (bounded by max_iters)
+    // a pass of the documented bound is 64 columns, two chunks
+    const int64_t max_iters = 2 * (vo.max_passes > 0 ? min(vo.max_passes, (int64_t)1 << 61) : kMaxIters);
     int base = 0;
-    uint64_t Pv[W1], Mv[W1];
+    uint32_t P[W], M[W];
 #pragma unroll
-    for (int v = 0; v < W1; v++) { Pv[v] = 0; Mv[v] = 0; }
-    // Peq word k (of x or of reversed x) into ring slot `slot` and its twin
-    auto build_word = [&](int slot, int64_t k) {
-        bd_build<B, R2>(ring, T_, slot, xc, m, k, rev, alpha);
-        for (uint32_t c = 0; c < alpha; c++)
-            ring[(size_t)(c * R2 + slot + R) * T_] = ring[(size_t)(c * R2 + slot) * T_];
-    };
+    for (int v = 0; v < W; v++) { P[v] = 0; M[v] = 0; }
 
     while (true) {
         if (++iters > max_iters) {
@@ -295,27 +341,24 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
                             }
                         } else {
                             const int32_t n1 = n / 2;
-                            ncols = rev ? n - n1 : n1;
-                            xc = a_long ? pa : pb;
+                            const int32_t nh = rev ? n - n1 : n1;
+                            ncols = (n - n1 + 31) & ~31;
+                            pad = ncols - nh;
+                            x64 = reinterpret_cast<const uint64_t *>(a_long ? pa : pb);
                             y64 = reinterpret_cast<const uint64_t *>(a_long ? pb : pa);
                             ywords = 2 * chunks_for(n, B);
-                            for (int wi = 0; wi < W1; wi++) build_word(wi, wi);
-#pragma unroll
-                            for (int v = 0; v < W1; v++) {
-                                Pv[v] = ~0ull;
-                                Mv[v] = 0ull;
-                            }
                             // the pair's band (see the head of this file); m - n <= kp here
-                            const int32_t klo = (kp - (m - n)) >> 1, khi = (kp + (m - n)) >> 1;
+                            klo = (kp - (m - n)) >> 1;
+                            const int32_t khi = (kp + (m - n)) >> 1;
                             wpair = (klo + khi + 64) >> 6;
+                            for (int wi = 0; wi <= W; wi++)
+                                pq_build<B, R>(ring, T_, wi, x64, m, (int64_t)(32 * wi) - klo - pad, pad, rev, alpha);
+                            diag_init<W>(P, M, klo);
+                            T = klo;
                             base = 0;
-                            k0 = 0;
-                            Tacc = 0;
-                            jbase = 1 - ((smove - klo) & 63);   // column 1 at chunk position s0
-                            snext = sym_word((int64_t)jbase - 1);
-                            next_move = klo + 1 + 64;
+                            j0 = 0;
+                            snext = sym_word(0);
                             rejected = false;
-                            budget = (ncols >> 6) + 4;
                             have = true;
                         }
                     }
@@ -324,195 +367,54 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         }
         if (!__any_sync(FULL, have)) break;
 
-        // one chunk: columns jbase .. jbase+63 of every active slot
-        int32_t lim = (have && !rejected) ? ncols - jbase : -1;   // steps s <= lim are columns of the pair
-        const int32_t slo = 1 - jbase;                             // and steps s >= slo (first chunk)
-        // symbols of y (forward) or of reversed y, 64/B per word; the word after
-        // the current one is requested one word ahead (snext: requested at the
-        // previous chunk's last word, or at the pair's start)
-        uint64_t sreg = 0;
-        // steps s_begin .. s_end-1; GUARD: only the steps that are columns of the
-        // lane's pair (without it every lane advances: lanes without a running
-        // pair compute values that nothing reads)
-        auto run_cols = [&](int s_begin, int s_end, auto guard) {
-            constexpr bool GUARD = decltype(guard)::value;
-#pragma unroll 2
-            for (int s = s_begin; s < s_end; s++) {
-                if ((s & (SPW - 1)) == 0) {
-                    const uint64_t v = sym_join(snext);
-                    sreg = rev ? sym_reverse<B>(v) : v;
-                    snext = sym_word((int64_t)jbase - 1 + s + SPW);
-                }
-                uint32_t c = (uint32_t)(sreg & CMASK);
+        // one chunk: columns j0 + 1 .. j0 + 32 of every slot
+        if (have && j0 > 0) {
+            // the word that left the window makes room for the one that enters
+            pq_build<B, R>(ring, T_, base, x64, m, (int64_t)j0 + 32 * W - klo - pad, pad, rev, alpha);
+            base = base + 1 == R ? 0 : base + 1;
+        }
+        const uint32_t *wrow = ring + base * T_;   // symbol 0's words of the window
+        uint32_t tacc = 0;
+#pragma unroll 1
+        for (int g = 0; g < 32; g += SPW) {
+            const uint64_t sv = sym_join(snext);
+            uint64_t sreg = rev ? sym_reverse<B>(sv) : sv;
+            snext = sym_word(j0 + g + SPW);
+#pragma unroll(W <= 4 ? 8 : 4)
+            for (int t = 0; t < SPW; t++) {
+                const uint32_t c = (uint32_t)sreg & CMASK;   // < alpha: packed codes, or 0 outside the string
                 sreg >>= B;
-                c = c < cmax ? c : cmax;
-                if (!GUARD || (s <= lim && s >= slo)) {
-                    const uint64_t *row = ring + ((size_t)c * R2 + base) * T_;   // the window's words
-                    uint64_t Eq[W1], A[W1], S[W1];
-#pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        Eq[v] = row[v * T_];
-                        A[v] = Eq[v] & Pv[v];
-                    }
-                    add_chain<W1>(S, A, Pv);
-                    uint64_t Ph[W1], Mh[W1];
-#pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        const uint64_t Xh = (S[v] ^ Pv[v]) | Eq[v];
-                        Ph[v] = Mv[v] | ~(Xh | Pv[v]);
-                        Mh[v] = Pv[v] & Xh;
-                    }
-#pragma unroll
-                    for (int v = W1 - 1; v >= 0; v--) {
-                        const uint64_t inP = (v > 0) ? (Ph[v > 0 ? v - 1 : 0] >> 63) : 1ull;
-                        const uint64_t inM = (v > 0) ? (Mh[v > 0 ? v - 1 : 0] >> 63) : 0ull;
-                        Ph[v] = (Ph[v] << 1) | inP;
-                        Mh[v] = (Mh[v] << 1) | inM;
-                    }
-#pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        const uint64_t X = Eq[v] | Mv[v];
-                        Pv[v] = Mh[v] | ~(X | Ph[v]);
-                        Mv[v] = Ph[v] & X;
-                    }
-                }
-            }
-        };
-        // LEAN (launches set by their longest pairs): a range of steps runs
-        // unguarded when every lane with a running pair has all its columns in
-        // it (most chunks of long pairs); with many pairs per slot the second
-        // copy of the loop costs more in instruction fetch than the guard
-        auto run_range = [&](int a, int b) {
-            if constexpr (LEAN) {
-                const bool whole = !(have && !rejected) || (slo <= a && lim >= b - 1);
-                if (__all_sync(FULL, whole)) {
-                    run_cols(a, b, std::false_type{});
-                    return;
-                }
-            }
-            run_cols(a, b, std::true_type{});
-        };
-        run_range(0, smove);
-        {
-            // window move before column j = jbase + smove, then the joint bound
-            const int32_t j = jbase + smove;
-            // every pair still running takes part in the joint bound, also before
-            // its first window move (short pairs have none)
-            const bool active = have && !rejected && j >= 1 && j <= ncols;
-            const bool moving = active && j == next_move;
-            int32_t lb = 0;
-            if (moving) {
-                next_move += 64;
-                Tacc += __popcll(Pv[0]) - __popcll(Mv[0]);
-#pragma unroll
-                for (int v = 0; v + 1 < W1; v++) { Pv[v] = Pv[v + 1]; Mv[v] = Mv[v + 1]; }
-                Pv[W1 - 1] = ~0ull;
-                Mv[W1 - 1] = 0ull;
-                k0++;
-                base = (base + 1 == R) ? 0 : base + 1;
-                {
-                    const int sl = base + W1 - 1;
-                    build_word(sl >= R ? sl - R : sl, k0 + W1 - 1);
-                }
-            }
-            if (active) {
-                // minimum over the window at column j-1; row 64*k0 (value T) takes part
-                int32_t run = 0, mn = 0;
-#pragma unroll
-                for (int v = 0; v < W1; v++) {
-#pragma unroll
-                    for (int q = 0; q < 16; q++) {
-                        const uint32_t idx = (uint32_t)((Pv[v] >> (4 * q)) & 15u) |
-                                             ((uint32_t)((Mv[v] >> (4 * q)) & 15u) << 4);
-                        const int32_t cand = run + s_nmin[idx];
-                        mn = cand < mn ? cand : mn;
-                        run += s_nsum[idx];
-                    }
-                }
-                lb = Tacc + (j - 1) + mn;
-            }
-            const int32_t lb_other = __shfl_xor_sync(FULL, lb, 1);
-            if (active && lb + lb_other > kp) {
-                rejected = true;
-                rej_col = j;
-                lim = -1;
+                diag_step<W>(P, M, tacc, wrow + (size_t)c * (R2 * T_), T_, (uint32_t)(g + t));
             }
         }
-        run_range(smove, 64);
-        jbase += 64;
-        if (have && --budget < 0 && !rejected && jbase <= ncols) {
-            // cannot happen for a consistent state: stop this pair and report it
-            pair_err(sg, (uint32_t)DERR_GUARD);
-            rejected = true;
-            rej_col = jbase;
+        T += 32 - __popc(tacc);
+        j0 += 32;
+        if ((iters & 1) == 0) {   // the joint bound
+            const int32_t lb = T + diag_min<W>(P, M, s_tab);
+            const int32_t lb_other = __shfl_xor_sync(FULL, lb, 1);
+            if (have && j0 < ncols && lb + lb_other > kp) rejected = true;
         }
 
-        // finished pairs: both halves done (all columns run, or rejected)
-        const bool lane_done = have && (rejected || jbase > ncols);
-        // every lane takes part in the shuffle (a short-circuit here would leave
-        // the warp's other lanes waiting at a different collective)
-        const int partner_done = __shfl_xor_sync(FULL, lane_done ? 1 : 0, 1);
-        const bool pair_done = lane_done && partner_done != 0;
+        // finished pairs: all columns run, or rejected (both lanes agree)
+        const bool pair_done = have && (rejected || j0 >= ncols);
         if (__any_sync(FULL, pair_done)) {
-            const int32_t T = Tacc + (rejected ? rej_col - 1 : ncols);
             if (pair_done) {
-                const unsigned long long cols = (unsigned long long)(rejected ? rej_col - 1 : ncols);
+                const int32_t real = j0 - pad;
+                const unsigned long long cols = real > 0 ? (unsigned long long)real : 0ull;
                 if (segs) atomicAdd(&wk[2 * sg + 1], cols * (unsigned long long)wpair);
                 else loc_cols += cols * (unsigned long long)wpair;
-#pragma unroll
-                for (int v = 0; v < W1; v++) {
-                    ring[(size_t)(2 * v) * T_] = Pv[v];
-                    ring[(size_t)(2 * v + 1) * T_] = Mv[v];
-                }
-                ring[(size_t)(2 * W1) * T_] = (uint64_t)(uint32_t)T | ((uint64_t)k0 << 32);
-                ring[(size_t)(2 * W1 + 1) * T_] = rejected ? 1ull : 0ull;
+                if (!rejected) diag_dump<W>(ring, T_, P, M, T);
             }
             __syncwarp();
+            int32_t ed = INT_MAX;                           // the distance when <= kp
+            if (pair_done && !rejected) {
+                const uint32_t *f = pq_smem + (threadIdx.x & ~1u);   // forward half's dump, then the backward one's
+                ed = diag_meet<W>(f, f + 1, T_, m, n / 2, n - n / 2, klo, rev ? 1 : 0);
+            }
+            ed = min(ed, __shfl_xor_sync(FULL, ed, 1));
             if (pair_done && !rev) {
-                bool pass = false;
-                int32_t ed = INT_MAX;                           // the distance when <= kp
-                const uint64_t *rb = smem + threadIdx.x + 1;   // backward half's dump
-                const bool rej_b = rb[(size_t)(2 * W1 + 1) * T_] != 0ull;
-                if (!rejected && !rej_b) {
-                    const uint64_t tb = rb[(size_t)(2 * W1) * T_];
-                    const int32_t Tb = (int32_t)(uint32_t)(tb & 0xFFFFFFFFull);
-                    const int64_t k0b = (int64_t)(tb >> 32);
-                    const int64_t k0f = k0;
-                    const uint64_t *rf = ring;
-                    // forward rows [64 k0f, min(m, 64(k0f+W1))]; backward row i' is row m - i'
-                    const int64_t f_hi = min((int64_t)m, 64 * (k0f + W1));
-                    const int64_t b_hi = min((int64_t)m, 64 * (k0b + W1));
-                    const int64_t i_lo = max(64 * k0f, (int64_t)m - b_hi);
-                    const int64_t i_hi = min(f_hi, (int64_t)m - 64 * k0b);
-                    if (i_lo <= i_hi) {
-                        auto prefix = [&](const uint64_t *dump, int64_t k0x, int32_t Tx, int64_t rowx) -> int32_t {
-                            int32_t acc = Tx;
-                            const int64_t nrows = rowx - 64 * k0x;
-                            for (int v = 0; v < W1; v++) {
-                                const int64_t lo = 64ll * v;
-                                if (lo >= nrows) break;
-                                const uint64_t msk = (nrows - lo >= 64) ? ~0ull : ((1ull << (nrows - lo)) - 1ull);
-                                acc += __popcll(dump[(size_t)(2 * v) * T_] & msk) -
-                                       __popcll(dump[(size_t)(2 * v + 1) * T_] & msk);
-                            }
-                            return acc;
-                        };
-                        int32_t F = prefix(rf, k0f, T, i_lo);
-                        int32_t Bv = prefix(rb, k0b, Tb, (int64_t)m - i_lo);
-                        int32_t best = F + Bv;
-                        for (int64_t i = i_lo; i < i_hi; i++) {
-                            const int64_t rf_ = i - 64 * k0f;                 // bit of row i+1 in the forward window
-                            const int64_t rb_ = (int64_t)m - i - 64 * k0b - 1; // bit of row m-i in the backward window
-                            const uint64_t fp = rf[(size_t)(2 * (rf_ >> 6)) * T_], fm = rf[(size_t)(2 * (rf_ >> 6) + 1) * T_];
-                            const uint64_t bp = rb[(size_t)(2 * (rb_ >> 6)) * T_], bm = rb[(size_t)(2 * (rb_ >> 6) + 1) * T_];
-                            F += (int32_t)((fp >> (rf_ & 63)) & 1ull) - (int32_t)((fm >> (rf_ & 63)) & 1ull);
-                            Bv -= (int32_t)((bp >> (rb_ & 63)) & 1ull) - (int32_t)((bm >> (rb_ & 63)) & 1ull);
-                            best = min(best, F + Bv);
-                        }
-                        pass = best <= kp;
-                        if (pass) ed = best;
-                    }
-                }
+                const bool pass = ed <= kp;
+                if (!pass) ed = INT_MAX;
                 if (uni) emit_union(p, umk, ed);
                 else emit(sg, p, pass);
             }
@@ -538,66 +440,56 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     }
 }
 
-template <int W1, int B, int TPB, bool LEAN>
+template <int W, int B, int TPB>
 cudaError_t launch_pq_tt(const uint4 *packed, const uint64_t *pofs, const int32_t *lens, int64_t n, uint32_t alpha,
                          const uint64_t *pairs, int64_t np, int32_t K, int spw_force, int wps, VerifyOut vo,
                          cudaStream_t s) {
     constexpr int threads = TPB;
-    const size_t smem = pq_smem_bytes(W1, alpha, threads);
-    cudaError_t e = cudaFuncSetAttribute(verify_pq_kernel<W1, B, TPB, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = pq_smem_bytes(W, alpha, threads);
+    cudaError_t e = cudaFuncSetAttribute(verify_pq_kernel<W, B, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_pq_kernel<W1, B, TPB, LEAN>, threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_pq_kernel<W, B, TPB>, threads, smem);
     if (per_sm < 1) per_sm = 1;
     const int64_t blocks = (int64_t)sms * per_sm;
-    verify_pq_kernel<W1, B, TPB, LEAN><<<(unsigned)blocks, threads, smem, s>>>(packed, pofs, lens, n, alpha, pairs, np, K,
-                                                                     sms, spw_force, wps, vo);
+    verify_pq_kernel<W, B, TPB><<<(unsigned)blocks, threads, smem, s>>>(packed, pofs, lens, n, alpha, pairs, np, K,
+                                                                       sms, spw_force, wps, vo);
     note_launches(1);
     return cudaGetLastError();
 }
 
-template <int W1, int B>
-cudaError_t launch_pq_t(const uint4 *packed, const uint64_t *pofs, const int32_t *lens, int64_t n, uint32_t alpha,
-                        const uint64_t *pairs, int64_t np, int32_t K, int threads, int spw_force, int wps, VerifyOut vo,
-                        bool lean, cudaStream_t s) {
-    // the lean variant for 2-bit codes and 128 threads (the long-string shape);
-    // the other shapes keep the guarded loop only (build time)
-    if (threads == 128 && lean && B == 2)
-        return launch_pq_tt<W1, 2, 128, true>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s);
-    if (threads == 128)
-        return launch_pq_tt<W1, B, 128, false>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s);
-    if (threads == 32)
-        return launch_pq_tt<W1, B, 32, false>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s);
-    return cudaErrorInvalidValue;
-}
-
 }  // namespace
 
-size_t pq_smem_bytes(int W1, uint32_t alpha, int threads) {
-    const size_t R2 = 2 * ((size_t)W1 + 1);
-    const size_t per = alpha * R2 > (size_t)(2 * W1 + 2) ? alpha * R2 : (size_t)(2 * W1 + 2);
-    return per * sizeof(uint64_t) * (size_t)threads;
+size_t pq_smem_bytes(int W, uint32_t alpha, int threads) {
+    return (size_t)alpha * 2 * ((size_t)W + 1) * sizeof(uint32_t) * (size_t)threads;
 }
 
-int pq_threads_for(int W1, uint32_t alpha) {
-    if (pq_smem_bytes(W1, alpha, 128) <= 160 * 1024) return 128;
-    return pq_smem_bytes(W1, alpha, 32) <= 220 * 1024 ? 32 : 0;
+int pq_threads_for(int W, uint32_t alpha) {
+    if (W > PQ_MAX_WORDS) return 0;
+    if (pq_smem_bytes(W, alpha, 128) <= 160 * 1024) return 128;
+    // blocks of one warp only for alphabets of more than four symbols (the rings
+    // of up to four fit 128 threads at every W)
+    return pq_smem_bytes(W, alpha, 32) <= 220 * 1024 ? 32 : 0;
 }
 
-cudaError_t launch_verify_pq(int W1, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
+cudaError_t launch_verify_pq(int W, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
                              const int32_t *lens, int64_t n, uint32_t alpha, const uint64_t *pairs, int64_t np,
-                             int32_t K, VerifyOut vo, cudaStream_t s, bool lean) {
+                             int32_t K, VerifyOut vo, cudaStream_t s) {
     if (np == 0) return cudaGetLastError();
     if (!vo.queue || !vo.sm_tickets || (threads != 128 && threads != 32)) return cudaErrorInvalidValue;
-#define EJ_PQ(WW)                                                                                          \
-    if (W1 == WW) {                                                                                        \
-        if (B == 2) return launch_pq_t<WW, 2>(packed, pofs, lens, n, alpha, pairs, np, K, threads, spw_force, wps, vo, lean, s); \
-        return launch_pq_t<WW, 8>(packed, pofs, lens, n, alpha, pairs, np, K, threads, spw_force, wps, vo, lean, s);   \
+#define EJ_PQ(WW)                                                                                                  \
+    if (W == WW) {                                                                                                 \
+        if (B == 2 && threads == 128)                                                                              \
+            return launch_pq_tt<WW, 2, 128>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s);    \
+        if (B == 8 && threads == 128)                                                                              \
+            return launch_pq_tt<WW, 8, 128>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s);    \
+        if (B == 8) return launch_pq_tt<WW, 8, 32>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s); \
     }
-    EJ_PQ(2) EJ_PQ(3) EJ_PQ(4) EJ_PQ(5) EJ_PQ(6) EJ_PQ(7) EJ_PQ(8) EJ_PQ(9) EJ_PQ(10) EJ_PQ(11) EJ_PQ(12)
+    EJ_PQ(1) EJ_PQ(2) EJ_PQ(3) EJ_PQ(4) EJ_PQ(5) EJ_PQ(6) EJ_PQ(7) EJ_PQ(8) EJ_PQ(9) EJ_PQ(10) EJ_PQ(11) EJ_PQ(12)
+    EJ_PQ(16) EJ_PQ(24)
 #undef EJ_PQ
     return cudaErrorInvalidValue;
 }
