@@ -169,7 +169,8 @@ int ej_set_verify_config(ej_ctx *ctx, int lanes_per_pair, int words_per_lane, in
 
 /*
  * Failure detection (the paper has no counterpart): the persistent verifier
- * (ej_schedule.mode 1, and the merged launch of a batch) bounds the passes of
+ * (ej_schedule.mode 1, the merged launch of a batch, and the pairs that the
+ * shared-string verifier leaves to it) bounds the passes of
  * each warp's work loop, so that a kernel that could not finish its queue
  * stops instead of running on. When the bound runs out the kernel records it
  * and returns, and the call reports EJ_ERR_TIMEOUT; the context stays usable.
@@ -340,10 +341,11 @@ void ej_batch_destroy(ej_batch *batch);
  *     otherwise the grid-strided verifier. 2: always the grid-strided verifier
  *     (one pass over the pairs; a warp's slots start together and the warp ends
  *     with its slowest pair). 3: the shared-string verifier: the candidates are
- *     grouped by their longer string x into warp tasks of up to 16 pairs, and
- *     the warp keeps one ring of x's match masks per direction for all of them
- *     (built cooperatively, once per task), instead of one per lane (two lanes
- *     per pair, up to 12 words per lane). 0 (default): 1 when the strings' mean
+ *     grouped by their longer string x into warp tasks of up to 32 pairs, one
+ *     lane per pair, and the warp keeps one ring of x's match masks for all of
+ *     them (built cooperatively, once per task) instead of one per lane; pairs
+ *     that outlive the rest of their task are left to the persistent verifier.
+ *     0 (default): 1 when the strings' mean
  *     length is at least 2048 (long pairs, where refilling pays); else 3 for
  *     alphabets of more than 4 symbols (whose per-lane rings leave the
  *     grid-strided verifier one or two warps per SM) and 2 for the rest.

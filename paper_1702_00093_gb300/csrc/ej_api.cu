@@ -37,6 +37,12 @@ enum BufId {
     B_NUM
 };
 
+// Device counters of a join (B_JCOUNT): [0] raw pairs, [1] largest bucket, [2]
+// candidates, [3] output pairs, [4] band cells, [5] word columns, [6] queue of the
+// persistent verifier, [7] tasks of the shared-string verifier, [8] its pairs left
+// to the persistent one.
+constexpr size_t JCOUNT_LEN = 16;
+
 struct Buf {
     void *p = nullptr;
     size_t cap = 0;
@@ -732,8 +738,8 @@ int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const Verif
 // verifier leave one or two warps per SM): two lanes per pair, the band within
 // 12 words per lane, the warp's shared area within the block's budget.
 bool sx_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
-    const int W1 = sx_band(p->K).W1;
-    if (vc.G != 2 || W1 > 12 || sx_smem_bytes(W1, p->alphabet_size) > 220 * 1024) return false;
+    const int W = sx_band(p->K).W;
+    if (vc.G != 2 || W > SX_MAX_WORDS || sx_smem_bytes(W, p->alphabet_size) > 220 * 1024) return false;
     const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
     return ctx->sched.mode == 3 || (ctx->sched.mode == 0 && !long_pairs && p->alphabet_size > 4);
 }
@@ -747,11 +753,11 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
                  VerifySeg *defer = nullptr, bool emitted = false) {
     const int64_t n = pl.st.n, T = (int64_t)p->r * p->m;
     unsigned long long *cnt = nullptr;
-    CKS(ensure_t(ctx, B_JCOUNT, 8, &cnt));
+    CKS(ensure_t(ctx, B_JCOUNT, JCOUNT_LEN, &cnt));
     uint32_t *derr = (uint32_t *)ctx->bufs[B_DERR].p;
     uint64_t hsize = 1;
     while (hsize < 2 * cap) hsize <<= 1;
-    uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr;
+    uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr, *spare = nullptr;
     CKS(ensure_t(ctx, B_RAW, (size_t)cap, &raw));
     CKS(ensure_t(ctx, B_CAND, (size_t)cap, &cand));
     CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
@@ -762,7 +768,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     const int order = sx ? 5 : bs.any_order ? 2 : ctx->sched.order != 0 ? ctx->sched.order : (pq_threads > 0 ? 4 : 3);
     // emitted: the raw pairs and counters [0], [1] are already written (shared
     // buckets of a batch)
-    CK(cudaMemsetAsync(emitted ? cnt + 2 : cnt, 0, (emitted ? 6 : 8) * sizeof(unsigned long long), s));
+    CK(cudaMemsetAsync(emitted ? cnt + 2 : cnt, 0, (emitted ? JCOUNT_LEN - 2 : JCOUNT_LEN) * sizeof(unsigned long long), s));
     if (!sx) {   // the shared-string verifier's candidates are deduplicated by sorting
         CKS(ensure_t(ctx, B_HASH, (size_t)hsize, &table));
         CK(cudaMemsetAsync(table, 0xFF, hsize * sizeof(uint64_t), s));
@@ -800,7 +806,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
         CKS(ensure_t(ctx, B_GSTART, (size_t)nb + 1, &gstart));
         CKS(ensure(ctx, B_DG_TEMP, dedup_grouped_temp_bytes(cap), &dgt));
         CK(launch_dedup_grouped(raw, cand, cap, n, pl.lens, sb.nclass, sb.width, cnt, dgt, fbins, fstarts, gstart,
-                                &sorted_cand, s));
+                                &sorted_cand, &spare, s));
         cand = sorted_cand;
     } else if (order == 3 || order == 5) {
         // candidates ordered by their first string (a warp's pairs share it), or
@@ -842,9 +848,9 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     vo.max_passes = ctx->loop_bound;
     const VerifyConfig &vc = bs.vc;
     if (sx) {
-        // warp tasks of up to 16 candidates sharing their longer string and the
-        // class of their length difference
-        const int64_t tcap = (int64_t)(cap / 16) + nb + 1;
+        // warp tasks of candidates sharing their longer string and the class of
+        // their length difference
+        const int64_t tcap = (int64_t)(cap / (uint64_t)sx_task_pairs()) + nb + 1;
         uint32_t *tcount = nullptr;
         uint64_t *tstart = nullptr, *tasks = nullptr;
         void *tscan = nullptr;
@@ -854,8 +860,23 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
         CKS(ensure(ctx, B_SX_SCAN, scan_temp_bytes(nb + 1), &tscan));
         CK(launch_sx_tasks(fbins, fstarts, nb, tcount, tstart, cnt + 7, tscan, tasks, s));
         if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));
-        CK(launch_verify_sx(sb.W1, pl.packed, pl.pofs, pl.B, pl.lens, n, p->alphabet_size, cand, tasks, cnt + 7,
+        // pairs that outlive the rest of their task (similar strings) go to the
+        // persistent verifier, where that has a block size for them
+        const int pq_after = pq_threads_for(pq_words(p->K), p->alphabet_size);
+        if (pq_after > 0) {
+            vo.defer = spare;
+            vo.defer_count = cnt + 8;
+        }
+        CK(launch_verify_sx(sb.W, pl.packed, pl.pofs, pl.B, pl.lens, n, p->alphabet_size, cand, tasks, cnt + 7,
                             tcap, p->K, vo, s));
+        if (pq_after > 0) {
+            VerifyOut v2 = vo;
+            v2.defer = nullptr;
+            v2.np_dev = cnt + 8;
+            CK(launch_verify_pq(pq_words(p->K), pq_after, ctx->sched.slots_per_warp ? ctx->sched.slots_per_warp : 16,
+                                ctx->sched.warps_per_subpartition, pl.packed, pl.pofs, pl.B, pl.lens, n,
+                                p->alphabet_size, spare, (int64_t)cap, p->K, v2, s));
+        }
     } else {
     if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));
     if (pq_threads > 0)
@@ -879,7 +900,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
 int back_segment(ej_ctx *ctx, const ej_params *p, uint64_t cap, VerifySeg *seg) {
     unsigned long long *cnt = nullptr;
     uint64_t *cand = nullptr, *app = nullptr;
-    CKS(ensure_t(ctx, B_JCOUNT, 8, &cnt));
+    CKS(ensure_t(ctx, B_JCOUNT, JCOUNT_LEN, &cnt));
     CKS(ensure_t(ctx, B_CAND, (size_t)cap, &cand));
     CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
     *seg = VerifySeg{cand, cnt + 2, cap, p->K, app, cnt + 3, cap, cnt + 4, (uint32_t *)ctx->bufs[B_DERR].p};
@@ -1426,7 +1447,7 @@ int batch_shared_emit(ej_batch *b, BatchJoin &o) {
         if (&m != &o) CK(cudaStreamWaitEvent(o.side, m.keyed, 0));
         unsigned long long *cnt = nullptr;
         uint64_t *raw = nullptr;
-        CKS(ensure_t(m.sub, B_JCOUNT, 8, &cnt));
+        CKS(ensure_t(m.sub, B_JCOUNT, JCOUNT_LEN, &cnt));
         CKS(ensure_t(m.sub, B_RAW, (size_t)m.cap, &raw));
         CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), o.side));
         se.keys[k] = m.keys;
@@ -2020,7 +2041,7 @@ int ej_join_plus(ej_ctx *ctx, const ej_strings *S, const ej_params *p, int32_t d
     CKS(ensure_t(sub, B_BHEADS, (size_t)(H * TT), &bheads));
     CKS(ensure_t(sub, B_BNEXT, (size_t)(nq * TT), &bnext));
     CKS(ensure_t(sub, B_DERR, 8, &derr));
-    CKS(ensure_t(sub, B_JCOUNT, 8, &cnt));
+    CKS(ensure_t(sub, B_JCOUNT, JCOUNT_LEN, &cnt));
     CK(cudaMemsetAsync(derr, 0, 4, s));
     CK(cudaMemsetAsync(bkeys, 0xFF, H * TT * sizeof(uint64_t), s));
     CK(cudaMemsetAsync(bheads, 0xFF, H * TT * sizeof(uint32_t), s));

@@ -143,6 +143,11 @@ __device__ __forceinline__ void add_chain<12>(uint64_t (&S)[12], const uint64_t 
 // |{(a, b): 0 <= a < lx, 0 <= b < ly, |a - b| <= K}|, Ukkonen's band size.
 __device__ __forceinline__ unsigned long long band_cells(int64_t lx, int64_t ly, int64_t K) {
     if (lx <= 0 || ly <= 0) return 0ull;
+    if (lx < 16384 && ly < 16384 && K < 16384) {   // the same sums in 32 bits
+        const int32_t a = (int32_t)lx, b = (int32_t)ly, k = (int32_t)K;
+        const int32_t rows = min(a, b + k), t = min(rows, max(0, b - k)), u = max(0, rows - 1 - k);
+        return (uint32_t)(t * (t - 1) / 2 + t * (k + 1) + (rows - t) * b - u * (u + 1) / 2);
+    }
     const int64_t amax = min(lx - 1, ly - 1 + K);   // rows whose band range is non-empty
     if (amax < 0) return 0ull;
     const int64_t t = min(amax + 1, max((int64_t)0, ly - K));  // rows whose range ends at a+K

@@ -283,15 +283,15 @@ int count_bins();
 // Dedup by sorting, for the shared-string verifier: raw[0 .. counters[0]) (the
 // rest of cap is not read) is sorted by (longer string, class of the length
 // difference, other string) with the LSD radix sort (alt: cap entries), the
-// distinct pairs written in that order to *cand_out (raw or alt, the other
-// holding the sorted keys) and counted in counters[2]; per group g = x * nclass
+// distinct pairs written in that order to *cand_out (raw or alt; *free_out is the
+// other, cap entries that hold nothing any more) and counted in counters[2]; per group g = x * nclass
 // + class: bins[g] (nb + 1 uint32, cleared here) its count, ends[g] its end
 // offset (nb uint64), gstart (nb uint64) scratch. temp: dedup_grouped_temp_bytes.
 size_t dedup_grouped_temp_bytes(uint64_t cap);
 cudaError_t launch_dedup_grouped(uint64_t *raw, uint64_t *alt, uint64_t cap, int64_t n, const int32_t *lens,
                                  uint32_t nclass, uint32_t width, unsigned long long *counters, void *temp,
                                  uint32_t *bins, uint64_t *ends, uint64_t *gstart, uint64_t **cand_out,
-                                 cudaStream_t s);
+                                 uint64_t **free_out, cudaStream_t s);
 struct VerifySeg;
 // Union of the candidate lists of a merged launch's joins (segs[0 .. nseg)):
 // every distinct pair once in upairs, with the mask of the joins that list it
@@ -348,22 +348,24 @@ cudaError_t launch_dedup_by_first(const uint64_t *raw, uint64_t cap, uint64_t *t
                                   int64_t n, uint32_t *bins, uint64_t *starts, void *scan_tmp, uint64_t *cand,
                                   unsigned long long *counters, cudaStream_t s,
                                   const int32_t *longer_lens = nullptr);
-// Shared-string verifier (ej_verify_sx.cu): warp tasks of up to 16 candidates
-// that share their longer string and length-difference class, from the bins of
-// launch_dedup_by_first with longer_lens (nb = n * nclass bins; tcount nb+1
-// uint32, tstart nb+1 uint64, tasks up to candidates/16 + nb entries;
-// *ntasks_dev = their number), and the verifier.
-// sx_band(K): the verifier's window W1 and the class width and count that keep
-// a task's band within it: a task's length differences lie in one class of
-// width D, so its band (the diagonals a cost-K alignment of any of its pairs
-// can use) spans at most K + (D - 1)/2 + 1 diagonals; D uses the rows that
-// ceil((K + 1) / 64) words leave (at least 7, else one more word).
+// Shared-string verifier (ej_verify_sx.cu): warp tasks of up to sx_task_pairs()
+// candidates that share their longer string and length-difference class, from
+// the groups of launch_dedup_grouped (nb groups; tcount nb+1 uint32, tstart nb+1
+// uint64, tasks up to candidates/sx_task_pairs() + nb entries; *ntasks_dev =
+// their number), and the verifier.
+// sx_band(K): the verifier's window of W 32-bit words and the class width and
+// count that keep a task's band within it: a task's length differences lie in
+// one class of width D, so its band (the diagonals a cost-K alignment of any of
+// its pairs can use) spans at most K + (D - 1)/2 + 1 diagonals; D uses the rows
+// that ceil((K + 1) / 32) words leave (at least 7, else one more word).
 struct SxBand {
-    int W1;
+    int W;
     uint32_t width, nclass;
 };
+constexpr int SX_MAX_WORDS = 12;
 SxBand sx_band(int32_t K);
-size_t sx_smem_bytes(int W1, uint32_t alpha);
+int sx_task_pairs();
+size_t sx_smem_bytes(int W, uint32_t alpha);
 cudaError_t launch_sx_tasks(const uint32_t *bins, const uint64_t *ends, int64_t n, uint32_t *tcount, uint64_t *tstart,
                             unsigned long long *ntasks_dev, void *scan_tmp, uint64_t *tasks, cudaStream_t s);
 int small_sort_max();
@@ -431,6 +433,11 @@ struct VerifyOut {
     const uint32_t *umask;
     const unsigned long long *unp_dev;
     uint64_t ucap;
+    // Shared-string verifier: when set, pairs that outlive the rest of their task
+    // are appended here (room for every pair) and left to a second verifier;
+    // *defer_count (zeroed before the launch) counts them.
+    uint64_t *defer;
+    unsigned long long *defer_count;
 };
 
 constexpr int SM_TICKETS = 1024;
@@ -468,9 +475,10 @@ int pq_threads_for(int W, uint32_t alpha);   // 0 if no block size fits
 cudaError_t launch_verify_pq(int W, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
                              const int32_t *lens, int64_t n, uint32_t alpha, const uint64_t *pairs, int64_t np,
                              int32_t K, VerifyOut vo, cudaStream_t s);
-// Shared-string verifier (W1 = 2..12): the pairs of tasks[0 .. *ntasks_dev)
-// (at most ntasks_cap), each task up to 16 pairs sharing their longer string.
-cudaError_t launch_verify_sx(int W1, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
+// Shared-string verifier (W = 1..SX_MAX_WORDS): the pairs of tasks[0 .. *ntasks_dev)
+// (at most ntasks_cap), each task up to sx_task_pairs() pairs sharing their longer
+// string.
+cudaError_t launch_verify_sx(int W, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
                              uint32_t alpha, const uint64_t *pairs, const uint64_t *tasks,
                              const unsigned long long *ntasks_dev, int64_t ntasks_cap, int32_t K, VerifyOut vo,
                              cudaStream_t s);

@@ -791,7 +791,7 @@ size_t dedup_grouped_temp_bytes(uint64_t cap) {
 cudaError_t launch_dedup_grouped(uint64_t *raw, uint64_t *alt, uint64_t cap, int64_t n, const int32_t *lens,
                                  uint32_t nclass, uint32_t width, unsigned long long *counters, void *temp,
                                  uint32_t *bins, uint64_t *ends, uint64_t *gstart, uint64_t **cand_out,
-                                 cudaStream_t s) {
+                                 uint64_t **free_out, cudaStream_t s) {
     if (nclass < 1 || width < 1 || cap == 0) return cudaErrorInvalidValue;
     uint32_t yb = 1;
     while ((1ll << yb) < n) yb++;
@@ -835,6 +835,7 @@ cudaError_t launch_dedup_grouped(uint64_t *raw, uint64_t *alt, uint64_t cap, int
     group_ends_kernel<<<(unsigned)(gg > 4096 ? 4096 : (gg ? gg : 1)), 256, 0, s>>>(bins, gstart, nb, ends);
     note_launches(2);
     *cand_out = out;
+    *free_out = keys;
     return cudaGetLastError();
 }
 

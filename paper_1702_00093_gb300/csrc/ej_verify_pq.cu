@@ -202,7 +202,6 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
                                              // at slot k mod R and k mod R + R, so that the
                                              // window's words sit at consecutive slots
     constexpr int SPW = 64 / B;              // symbols per 64-bit word
-    constexpr uint32_t CMASK = (1u << B) - 1u;
     extern __shared__ uint32_t pq_smem[];
     __shared__ uint32_t s_tab[256];
     diag_fill_table(s_tab);
@@ -380,11 +379,20 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             const uint64_t sv = sym_join(snext);
             uint64_t sreg = rev ? sym_reverse<B>(sv) : sv;
             snext = sym_word(j0 + g + SPW);
-#pragma unroll(W <= 4 ? 8 : 4)
-            for (int t = 0; t < SPW; t++) {
-                const uint32_t c = (uint32_t)sreg & CMASK;   // < alpha: packed codes, or 0 outside the string
-                sreg >>= B;
-                diag_step<W>(P, M, tacc, wrow + (size_t)c * (R2 * T_), T_, (uint32_t)(g + t));
+            // four symbols per step; a 2-bit code is masked in place and its row's
+            // offset is one multiplication (CST is a multiple of 64)
+            constexpr uint32_t CST = R2 * T_ * sizeof(uint32_t);
+            const char *wbase = reinterpret_cast<const char *>(wrow);
+#pragma unroll(W <= 4 ? 2 : 1)
+            for (int t = 0; t < SPW; t += 4) {
+                const uint32_t sw = (uint32_t)sreg;
+                sreg >>= 4 * B;
+#pragma unroll
+                for (int q = 0; q < 4; q++) {   // codes are < alpha (0 outside the string)
+                    const uint32_t off = B == 2 ? (sw & (3u << (2 * q))) * (CST >> (2 * q))
+                                                : __byte_perm(sw, 0u, 0x4440 | q) * CST;
+                    diag_step<W>(P, M, tacc, reinterpret_cast<const uint32_t *>(wbase + off), T_, (uint32_t)(g + t + q));
+                }
             }
         }
         T += 32 - __popc(tacc);

@@ -1,36 +1,50 @@
 // Verifier for pairs grouped by their longer string (Section 3.3, the last loop
-// of Algorithm 3): the same exact test ED(x, y) <= K as the two-lane
-// block-aligned verifier, with the match masks of x shared by a warp.
+// of Algorithm 3): the same exact test ED(x, y) <= K, with the match masks of x
+// shared by a warp.
 //
 // The candidates arrive grouped by x, the longer string of each pair, and by
 // the class of the length difference d = |x| - |y| (sx_band), in warp tasks of
-// up to 16 pairs that all share x and the class. A warp runs its 16 pairs in
-// two lanes each (forward half and backward half, as in verify_bd_kernel).
-// A path of cost <= K of a pair stays on the diagonals i - j in
+// up to 32 pairs that all share x and the class, one lane per pair. A path of
+// cost <= K of a pair stays on the diagonals i - j in
 // [-floor((K - d)/2), floor((K + d)/2)] (the persistent verifier's band); the
 // task's band is the union of its pairs' bands, at most K + 1 + (D - 1)/2
-// diagonals for a class of width D. All pairs of a task start together and the
-// band window of every pair moves at the same columns (klo + 1 + 64t, klo the
-// task band's upper reach), so the windows of all forward halves cover the
-// same 64-row words of x, and those of all backward halves the same words of
-// reversed x: the warp keeps one ring of match masks per direction in
-// shared memory instead of one per lane. For large alphabets that is 16x less
-// shared memory per pair, which is what limited the per-lane verifier to one or
-// two warps per SM, and each word is built once per task, by the whole warp:
-// lane t takes rows t and t + 32, and __match_any_sync gives every symbol's
-// mask of the word in two steps.
+// diagonals for a class of width D, held in a diagonal window of W 32-bit words
+// (ej_diag.cuh). All pairs of a task start together, so at every column their
+// windows cover the same rows of x: the warp keeps one ring of W + 1 match words
+// per symbol in shared memory. A word is built by the whole warp, every 32
+// columns: lane t reads row t, one ballot per bit of the symbol codes gives the
+// rows' bit planes, and lane c combines them into symbol c's mask.
 //
-// Early exit every 32 columns is decided by both halves of a pair together
-// (the joint bound of the other verifiers), and the task ends when all of its
-// pairs are decided.
-#include "ej_bitpar.cuh"
+// One lane per pair rather than two (halves that meet in the middle): nearly all
+// of these candidates are rejected after the same number of columns (about
+// K / 0.7 for text, 2 K for DNA, in one half or summed over two), and one lane
+// per pair halves the tasks, and with them the rings, the loads and the window
+// minima per pair.
+//
+// Early exit. The window's minimum (ej_diag.cuh) is a lower bound of the
+// distance. It is taken first after 11 K / 8 columns, then when the growth so far
+// says that the slowest of the pairs about to be rejected will be (a multiple of
+// 8 columns). Pairs that are not (similar strings run to the end) would keep the
+// warp with most lanes idle: once at most 8 lanes are left and all of them are
+// such, they are appended to a list that the persistent verifier takes from the
+// start (vo.defer; without one the task runs to its end).
+//
+// What bounds it: 32-bit integer instructions, 10 W + about 8 per column and
+// lane, and 5 per window row and quarter for a minimum.
+// 20000 tasks a millisecond and more keep the integer pipe 79% busy (0.59
+// instructions issued a cycle). 622M candidates of 200000 protein-like strings
+// (K = 40, W = 2): 274 -> 77 ms against two lanes per pair on 64-bit block-aligned
+// words with a test every 32 columns; 30M of 120000 text-like strings (K = 200,
+// W = 7): 97.3 -> 41.7 ms and 3.4 ms for the pairs handed over.
+#include "ej_diag.cuh"
 
 namespace ej {
 
 namespace {
 
-constexpr int SX_WARPS = 4;    // warps per block
-constexpr int SX_CHECK = 32;   // columns between the joint early-exit tests (a power of two)
+constexpr int SX_WARPS = 4;       // warps per block
+constexpr int SX_PAIRS = 32;      // pairs per task
+constexpr int SX_DEFER_MAX = 8;   // lanes left when a task hands its similar pairs over
 
 // Symbol i (0 <= i < m) of a packed string.
 template <int B>
@@ -39,39 +53,41 @@ __device__ __forceinline__ uint32_t sym_at(const uint4 *__restrict__ xc, int64_t
     return (reinterpret_cast<const uint32_t *>(xc)[i >> 4] >> (2 * (uint32_t)(i & 15))) & 3u;
 }
 
-// Word k (rows 64k+1 .. 64k+64) of x, or of reversed x, built by the whole warp
-// into ring slot `slot` (entry c * RS + slot for symbol c): lane t reads rows t
-// and t + 32 (coop_load), and the lanes holding the same symbol find one
-// another with __match_any_sync, which is that symbol's mask of the 32 rows
-// (coop_store). The loads of several words are issued before any of them is
-// stored, so that their latencies overlap.
-struct WordSyms {
-    uint32_t s0, s1;
-};
-
+// Row t of a match word whose row 0 is symbol i0 - t of x: its code, or
+// NO_SYMBOL outside x.
+constexpr uint32_t NO_SYMBOL = 0x100u;
 template <int B>
-__device__ __forceinline__ WordSyms coop_load(const uint4 *__restrict__ xc, int64_t m, int64_t k, bool rev, int lane) {
-    const int64_t i0 = rev ? m - 1 - 64 * k - lane : 64 * k + lane;
-    const int64_t i1 = rev ? i0 - 32 : i0 + 32;
-    WordSyms w;
-    w.s0 = (i0 >= 0 && i0 < m) ? sym_at<B>(xc, i0) : 0xFFFFu;
-    w.s1 = (i1 >= 0 && i1 < m) ? sym_at<B>(xc, i1) : 0xFFFFu;
-    return w;
+__device__ __forceinline__ uint32_t row_sym(const uint4 *__restrict__ xc, int32_t m, int64_t i) {
+    return i >= 0 && i < m ? sym_at<B>(xc, i) : NO_SYMBOL;
 }
 
-__device__ __forceinline__ void coop_store(uint64_t *ring, int RS, int slot, WordSyms w, uint32_t alpha, int lane) {
-    const unsigned m0 = __match_any_sync(FULL, w.s0);
-    const unsigned m1 = __match_any_sync(FULL, w.s1);
-    for (uint32_t c = lane; c < alpha; c += 32) ring[(size_t)c * RS + slot] = 0ull;
-    __syncwarp();
-    // lanes with the same symbol write the same value
-    if (w.s0 < alpha) reinterpret_cast<uint32_t *>(ring + (size_t)w.s0 * RS + slot)[0] = m0;
-    if (w.s1 < alpha) reinterpret_cast<uint32_t *>(ring + (size_t)w.s1 * RS + slot)[1] = m1;
-    __syncwarp();
+// The word of the rows' symbols (lane t: row t) for every symbol, into ring
+// entries c * RS + slot and, R entries further, their twins (so that a window's
+// words sit at consecutive entries from any slot on).
+__device__ __forceinline__ void sx_build(uint32_t *ring, int RS, int R, int slot, uint32_t sym, uint32_t alpha, int planes,
+                                         int lane) {
+    const uint32_t valid = __ballot_sync(FULL, sym != NO_SYMBOL);
+    uint32_t bp[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+        if (k < planes) bp[k] = __ballot_sync(FULL, (sym >> k) & 1u);
+    for (uint32_t c = lane; c < alpha; c += 32) {
+        uint32_t e = valid;
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (k < planes) e &= ((c >> k) & 1u) ? bp[k] : ~bp[k];
+        ring[(size_t)c * RS + slot] = e;
+        ring[(size_t)c * RS + slot + R] = e;
+    }
 }
 
-template <int W1, int B>
-__global__ void __launch_bounds__(SX_WARPS * 32, 4)
+template <int W>
+constexpr int sx_blocks() {   // resident blocks per SM the registers are limited to
+    return W <= 3 ? 5 : W <= 8 ? 4 : 3;
+}
+
+template <int W, int B>
+__global__ void __launch_bounds__(SX_WARPS * 32, sx_blocks<W>())
 verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ pofs,
                  const int32_t *__restrict__ lens, int64_t n_str, uint32_t alpha,
                  const uint64_t *__restrict__ pairs, const uint64_t *__restrict__ tasks,
@@ -79,33 +95,18 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
                  int32_t warp_words, VerifyOut vo) {
     uint32_t *__restrict__ err = vo.err;
     unsigned long long *__restrict__ work = vo.work;
-    extern __shared__ uint64_t smem[];
-    __shared__ int8_t s_nsum[256];
-    __shared__ int8_t s_nmin[256];
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
-        const uint32_t P = t & 15u, M = t >> 4;
-        int run = 0, mn = 1 << 20;
-        for (int k = 0; k < 4; k++) {
-            run += (int)((P >> k) & 1u) - (int)((M >> k) & 1u);
-            mn = run < mn ? run : mn;
-        }
-        s_nsum[t] = (int8_t)run;
-        s_nmin[t] = (int8_t)mn;
-    }
+    constexpr int R = W + 1;
+    extern __shared__ uint32_t sx_smem[];
+    __shared__ uint32_t s_tab[256];
+    diag_fill_table(s_tab);
     __syncthreads();
-    constexpr int R = W1;   // ring slots: the new bottom word takes the dropped top word's slot
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    uint64_t *wbase = smem + (size_t)wib * warp_words;
-    uint64_t *ringF = wbase;                          // words of x
-    uint64_t *ringB = wbase + (size_t)alpha * RS;     // words of reversed x
-    uint64_t *dump = wbase;                           // after a task's columns: entry e of lane L at e*32+L
-    const bool rev = lane & 1;
-    const int slot_pair = lane >> 1;
-    uint64_t *myring = rev ? ringB : ringF;
+    uint32_t *ring = sx_smem + (size_t)wib * warp_words;
     const int64_t cap_t = (int64_t)*ntasks_dev;
     const int64_t ntasks = cap_t < ntasks_cap ? cap_t : ntasks_cap;
     const int64_t nw = (int64_t)gridDim.x * SX_WARPS;
+    const int planes = alpha <= 1 ? 1 : 32 - __clz(alpha - 1u);
 
     unsigned long long loc_cells = 0, loc_cols = 0;
     // a task's descriptor and this lane's pair are loaded during the task before
@@ -113,24 +114,23 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     uint64_t tk_next = 0, pr_next = 0;
     if (t < ntasks) {
         tk_next = tasks[t];
-        if (slot_pair < (int)(tk_next & 31u)) pr_next = pairs[(int64_t)(tk_next >> 5) + slot_pair];
+        if (lane < (int)(tk_next & 63u)) pr_next = pairs[(int64_t)(tk_next >> 6) + lane];
     }
     for (; t < ntasks; t += nw) {   // warp-uniform
         const uint64_t tk = tk_next;
         const uint64_t pr = pr_next;
         if (t + nw < ntasks) {
             tk_next = tasks[t + nw];
-            if (slot_pair < (int)(tk_next & 31u)) pr_next = pairs[(int64_t)(tk_next >> 5) + slot_pair];
+            if (lane < (int)(tk_next & 63u)) pr_next = pairs[(int64_t)(tk_next >> 6) + lane];
         }
-        const int64_t first = (int64_t)(tk >> 5);
-        const int cnt = (int)(tk & 31u);
-        bool valid = slot_pair < cnt;
+        const int64_t first = (int64_t)(tk >> 6);
+        bool valid = lane < (int)(tk & 63u);
         int64_t a = 0, b = 0;
         if (valid) {
             a = (int64_t)(pr >> 32);
             b = (int64_t)(pr & 0xFFFFFFFFull);
             if (a >= n_str || b >= n_str) {
-                if (!rev) atomicOr(err, (uint32_t)DERR_PAIR);
+                atomicOr(err, (uint32_t)DERR_PAIR);
                 valid = false;
             }
         }
@@ -141,211 +141,177 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         // every pair of a task has the same x (its first pair's)
         const int64_t xs = __shfl_sync(FULL, valid ? xi : -1, 0);
         if (valid && xi != xs) {
-            if (!rev) atomicOr(err, (uint32_t)DERR_GUARD);
+            atomicOr(err, (uint32_t)DERR_GUARD);
             valid = false;
         }
-        bool decided = !valid, pass = false;
-        if (valid && m - n > K) decided = true;
-        else if (valid && n == 0) { decided = true; pass = m <= K; }
-        const int32_t n1 = n / 2;
-        const int32_t ncols = decided ? 0 : (rev ? n - n1 : n1);
-        const int32_t maxcols = (int32_t)__reduce_max_sync(FULL, (unsigned)ncols);
+        bool running = valid, pass = false, deferred = false;
+        if (valid && m - n > K) running = false;
+        else if (valid && n == 0) { running = false; pass = m <= K; }
+        int32_t cols_run = 0;
         // the task's band: the diagonals a cost-K alignment of any of its
         // undecided pairs can use (their length differences lie in one class)
-        const unsigned nlo = __reduce_min_sync(FULL, decided ? 0xFFFFFFFFu : (unsigned)n);
-        const unsigned nhi = __reduce_max_sync(FULL, decided ? 0u : (unsigned)n);
-
-        uint64_t Pv[W1], Mv[W1];
-#pragma unroll
-        for (int v = 0; v < W1; v++) { Pv[v] = ~0ull; Mv[v] = 0ull; }
-        int32_t T = 0, cols_run = 0;
-        int64_t k0 = 0;
-        bool rejected = false;
-        if (maxcols > 0) {
-            const int32_t mx = xs >= 0 ? lens[xs] : 0;
-            const uint4 *xc = packed + pofs[xs >= 0 ? xs : 0];
-            // the first W1 words of both directions, loaded four words at a time
-#pragma unroll
-            for (int w0 = 0; w0 < W1; w0 += 2) {
-                WordSyms f[2], r[2];
-#pragma unroll
-                for (int d = 0; d < 2; d++) {
-                    if (w0 + d < W1) {
-                        f[d] = coop_load<B>(xc, mx, w0 + d, false, lane);
-                        r[d] = coop_load<B>(xc, mx, w0 + d, true, lane);
-                    }
-                }
-#pragma unroll
-                for (int d = 0; d < 2; d++) {
-                    if (w0 + d < W1) {
-                        coop_store(ringF, RS, w0 + d, f[d], alpha, lane);
-                        coop_store(ringB, RS, w0 + d, r[d], alpha, lane);
-                    }
-                }
-            }
-            SymReader<B> yf;
-            SymReaderRev<B> yb;
-            if (!decided) {
-                if (rev) yb.init(packed + pofs[yi], n);
-                else yf.init(packed + pofs[yi], chunks_for(n1, B));
-            }
-            const uint32_t cmax = alpha - 1u;
-            int base = 0;              // ring slot of the window's top word (the same for the whole warp)
-            int64_t kr = 0;            // window moves of the warp so far
+        const unsigned nlo = __reduce_min_sync(FULL, running ? (unsigned)n : 0xFFFFFFFFu);
+        const unsigned nhi = __reduce_max_sync(FULL, running ? (unsigned)n : 0u);
+        if (nhi > 0) {   // some pair is running
+            const int32_t mx = lens[xs];
+            const uint4 *xc = packed + pofs[xs];
             const int32_t klo = (K - (mx - (int32_t)nhi)) >> 1, khi = (K + (mx - (int32_t)nlo)) >> 1;
-            if (klo + khi + 64 > 64 * W1 && lane == 0) atomicOr(err, (uint32_t)DERR_GUARD);   // not by construction
-            int32_t next_move = klo + 1 + 64;   // the window moves down before the columns klo + 1 + 64t
-            bool done = decided;
-            for (int32_t j = 1; j <= maxcols; j++) {
-                if ((j & (SX_CHECK - 1)) == 0) {
-                    // joint early exit at column j-1 of both halves (j <= n1 <= n - n1)
-                    const bool chk = !done && j <= n1;
-                    int32_t lb = 0;
-                    if (chk) {
-                        int32_t run = 0, mn = 0;
-#pragma unroll
-                        for (int v = 0; v < W1; v++) {
-#pragma unroll
-                            for (int q = 0; q < 16; q++) {
-                                const uint32_t idx = (uint32_t)((Pv[v] >> (4 * q)) & 15u) |
-                                                     ((uint32_t)((Mv[v] >> (4 * q)) & 15u) << 4);
-                                const int32_t cand = run + s_nmin[idx];
-                                mn = cand < mn ? cand : mn;
-                                run += s_nsum[idx];
-                            }
-                        }
-                        lb = T + mn;
+            if (klo + khi + 1 > 32 * W && lane == 0) atomicOr(err, (uint32_t)DERR_GUARD);   // not by construction
+            // y, forward from its first chunk, a load ahead of its use: 16 columns
+            // (B = 8) or 32 (B = 2) per load
+            const char *yp = reinterpret_cast<const char *>(packed + (running ? pofs[yi] : 0));
+            const uint32_t ybytes = running ? 16u * (uint32_t)chunks_for(n, B) : 0u;
+            constexpr uint32_t YB = B == 8 ? 16 : 8;   // bytes per load
+            auto y_load = [&](uint32_t off) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (off < ybytes) {
+                    if (B == 8) {
+                        v = *reinterpret_cast<const uint4 *>(yp + off);
+                    } else {
+                        const uint2 h = *reinterpret_cast<const uint2 *>(yp + off);
+                        v.x = h.x;
+                        v.y = h.y;
                     }
-                    const int32_t lb_other = __shfl_xor_sync(FULL, lb, 1);
-                    if (chk && lb + lb_other > K) {
-                        rejected = true;
-                        done = true;
-                        cols_run = j - 1;
-                    }
-                    if (__all_sync(FULL, done || j > ncols)) break;
                 }
-                const bool running = !done && j <= ncols;
-                if (j == next_move) {   // warp-uniform
-                    next_move += 64;
-                    if (running) {
-                        // drop the top word into T, shift the window down one word
-                        T += __popcll(Pv[0]) - __popcll(Mv[0]);
+                return v;
+            };
+            uint4 ynext = y_load(0), ycur = ynext;
+            uint32_t yoff = YB;
+            uint32_t P[W], M[W];
+            diag_init<W>(P, M, klo);
+            int32_t T = klo;
+            // the first W + 1 words of x, and the rows of the next one
+            {
+                uint32_t sy[W + 1];
 #pragma unroll
-                        for (int v = 0; v + 1 < W1; v++) { Pv[v] = Pv[v + 1]; Mv[v] = Mv[v + 1]; }
-                        Pv[W1 - 1] = ~0ull;
-                        Mv[W1 - 1] = 0ull;
-                        k0++;
-                    }
-                    kr++;
-                    const int freed = base;   // the dropped top word's slot takes the new bottom word
-                    base = (base + 1 == R) ? 0 : base + 1;
-                    const WordSyms f = coop_load<B>(xc, mx, kr + W1 - 1, false, lane);
-                    const WordSyms r = coop_load<B>(xc, mx, kr + W1 - 1, true, lane);
-                    coop_store(ringF, RS, freed, f, alpha, lane);
-                    coop_store(ringB, RS, freed, r, alpha, lane);
-                }
-                if (running) {
-                    uint32_t c;
-                    if (rev) { c = yb.code(); yb.advance(); }
-                    else { c = yf.code(); yf.advance(); }
-                    c = c < cmax ? c : cmax;   // codes of a validated string are < alpha
-                    const uint64_t *row = myring + (size_t)c * RS;
-                    uint64_t Eq[W1], A[W1], S[W1];
+                for (int w = 0; w <= W; w++) sy[w] = row_sym<B>(xc, mx, 32 * w - klo + lane);
+                __syncwarp();   // the ring of the task before is no longer read
 #pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        const int sl = base + v;
-                        Eq[v] = row[sl >= R ? sl - R : sl];
-                        A[v] = Eq[v] & Pv[v];
-                    }
-                    add_chain<W1>(S, A, Pv);
-                    uint64_t Ph[W1], Mh[W1];
-#pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        const uint64_t Xh = (S[v] ^ Pv[v]) | Eq[v];
-                        Ph[v] = Mv[v] | ~(Xh | Pv[v]);
-                        Mh[v] = Pv[v] & Xh;
-                    }
-#pragma unroll
-                    for (int v = W1 - 1; v >= 0; v--) {
-                        const uint64_t inP = (v > 0) ? (Ph[v > 0 ? v - 1 : 0] >> 63) : 1ull;
-                        const uint64_t inM = (v > 0) ? (Mh[v > 0 ? v - 1 : 0] >> 63) : 0ull;
-                        Ph[v] = (Ph[v] << 1) | inP;
-                        Mh[v] = (Mh[v] << 1) | inM;
-                    }
-#pragma unroll
-                    for (int v = 0; v < W1; v++) {
-                        const uint64_t X = Eq[v] | Mv[v];
-                        Pv[v] = Mh[v] | ~(X | Ph[v]);
-                        Mv[v] = Ph[v] & X;
-                    }
-                    T += 1;   // the row above the window: +1 per column
-                }
+                for (int w = 0; w <= W; w++) sx_build(ring, RS, R, w, sy[w], alpha, planes, lane);
+                __syncwarp();
             }
-            if (!decided && !rejected) cols_run = ncols;
-        }
-        // exchange through the warp's shared area (the rings are no longer read)
-        __syncwarp();
-#pragma unroll
-        for (int v = 0; v < W1; v++) {
-            dump[(size_t)(2 * v) * 32 + lane] = Pv[v];
-            dump[(size_t)(2 * v + 1) * 32 + lane] = Mv[v];
-        }
-        dump[(size_t)(2 * W1) * 32 + lane] = (uint64_t)(uint32_t)T | ((uint64_t)k0 << 32);
-        dump[(size_t)(2 * W1 + 1) * 32 + lane] = rejected ? 1ull : 0ull;
-        __syncwarp();
-        if (!rev && !decided) {
-            const uint64_t *rf = dump + lane, *rb = dump + lane + 1;
-            const bool rej_b = rb[(size_t)(2 * W1 + 1) * 32] != 0ull;
-            if (rejected || rej_b) {
-                pass = false;
-            } else {
-                const uint64_t tb = rb[(size_t)(2 * W1) * 32];
-                const int32_t Tb = (int32_t)(uint32_t)(tb & 0xFFFFFFFFull);
-                const int64_t k0b = (int64_t)(tb >> 32);
-                const int64_t k0f = k0;
-                const int64_t f_hi = min((int64_t)m, 64 * (k0f + W1));
-                const int64_t b_hi = min((int64_t)m, 64 * (k0b + W1));
-                const int64_t i_lo = max(64 * k0f, (int64_t)m - b_hi);
-                const int64_t i_hi = min(f_hi, (int64_t)m - 64 * k0b);
-                if (i_lo > i_hi) {
-                    pass = false;
+            uint32_t sym_next = row_sym<B>(xc, mx, (int64_t)32 * (W + 1) - klo + lane);
+            int base = 0;
+            int32_t j = 0;                                             // columns done
+            int32_t next_check = (11 * (K >> 3) + 15) & ~7;             // a multiple of 8, above K
+            if (next_check <= K) next_check = (K + 8) & ~7;
+            int32_t jend = (int32_t)nlo;                               // the first end of a running pair
+            while (true) {
+                if ((j & 31) == 0 && j > 0) {
+                    // the word that left the window makes room for the one that enters
+                    __syncwarp();
+                    sx_build(ring, RS, R, base, sym_next, alpha, planes, lane);
+                    base = base + 1 == R ? 0 : base + 1;
+                    sym_next = row_sym<B>(xc, mx, (int64_t)j + 32 * (W + 1) - klo + lane);
+                    __syncwarp();
+                }
+                // the symbols of 8 columns in two words (B = 8) or in the low half of one
+                uint32_t s0, s1 = 0;
+                if (B == 8) {
+                    if ((j & 15) == 0) {
+                        ycur = ynext;
+                        ynext = y_load(yoff);
+                        yoff += YB;
+                        s0 = ycur.x;
+                        s1 = ycur.y;
+                    } else {
+                        s0 = ycur.z;
+                        s1 = ycur.w;
+                    }
                 } else {
-                    // F(i) = value of row i at column n1 (forward), B(i) = value of
-                    // row m-i at column n-n1 (backward); ED = min_i F(i) + B(i)
-                    auto prefix = [&](const uint64_t *d, int64_t k0x, int32_t Tx, int64_t row) -> int32_t {
-                        int32_t acc = Tx;
-                        const int64_t nrows = row - 64 * k0x;
-                        for (int v = 0; v < W1; v++) {
-                            const int64_t lo = 64ll * v;
-                            if (lo >= nrows) break;
-                            const uint64_t msk = (nrows - lo >= 64) ? ~0ull : ((1ull << (nrows - lo)) - 1ull);
-                            acc += __popcll(d[(size_t)(2 * v) * 32] & msk) - __popcll(d[(size_t)(2 * v + 1) * 32] & msk);
-                        }
-                        return acc;
-                    };
-                    int32_t F = prefix(rf, k0f, T, i_lo);
-                    int32_t Bv = prefix(rb, k0b, Tb, (int64_t)m - i_lo);
-                    int32_t best = F + Bv;
-                    for (int64_t i = i_lo; i < i_hi; i++) {
-                        const int64_t rf_ = i - 64 * k0f;
-                        const int64_t rb_ = (int64_t)m - i - 64 * k0b - 1;
-                        const uint64_t fp = rf[(size_t)(2 * (rf_ >> 6)) * 32], fm = rf[(size_t)(2 * (rf_ >> 6) + 1) * 32];
-                        const uint64_t bp = rb[(size_t)(2 * (rb_ >> 6)) * 32], bm = rb[(size_t)(2 * (rb_ >> 6) + 1) * 32];
-                        F += (int32_t)((fp >> (rf_ & 63)) & 1ull) - (int32_t)((fm >> (rf_ & 63)) & 1ull);
-                        Bv -= (int32_t)((bp >> (rb_ & 63)) & 1ull) - (int32_t)((bm >> (rb_ & 63)) & 1ull);
-                        best = min(best, F + Bv);
+                    if ((j & 31) == 0) {
+                        ycur = ynext;
+                        ynext = y_load(yoff);
+                        yoff += YB;
                     }
-                    pass = best <= K;
+                    s0 = ((j & 16) ? ycur.y : ycur.x) >> ((j & 8) * 2);
                 }
+                const uint32_t *wrow = ring + base;
+                const uint32_t sh0 = (uint32_t)(j & 31);
+                uint32_t tacc = 0;
+                if (j + 8 < jend) {
+#pragma unroll(W <= 4 ? 2 : 1)
+                    for (int h = 0; h < 2; h++) {
+                        const uint32_t sw = B == 8 ? (h ? s1 : s0) : s0 >> (8 * h);   // the symbols of 4 columns
+#pragma unroll
+                        for (int q = 0; q < 4; q++) {
+                            const uint32_t c = B == 8 ? __byte_perm(sw, 0u, 0x4440 | q) : (sw >> (2 * q)) & 3u;
+                            diag_step<W>(P, M, tacc, wrow + c * (uint32_t)RS, 1, sh0 + 4 * h + q);
+                        }
+                    }
+                    T += 8 - __popc(tacc);
+                    j += 8;
+                    if (j < next_check) continue;
+                } else {
+                    // some pair ends within these columns: one at a time
+#pragma unroll 1
+                    for (int q = 0; q < 8; q++) {
+                        const uint32_t c = B == 8 ? ((q & 4 ? s1 : s0) >> (8 * (q & 3))) & 0xFFu : (s0 >> (2 * q)) & 3u;
+                        tacc = 0;
+                        diag_step<W>(P, M, tacc, wrow + c * (uint32_t)RS, 1, sh0 + q);
+                        T += 1 - (int32_t)(tacc >> 31);
+                        if (running && j + q + 1 == n) {
+                            // D(m, n): the row m is m - n + klo below the window's top
+                            int32_t cnt = 0;
+                            const int32_t rows = m - n + klo;
+#pragma unroll
+                            for (int v = 0; v < W; v++) {
+                                const int32_t left = rows - 32 * v;
+                                const uint32_t msk = left <= 0 ? 0u : left >= 32 ? ~0u : (1u << left) - 1u;
+                                cnt += __popc(P[v] & msk) - __popc(M[v] & msk);
+                            }
+                            pass = T + cnt <= K;
+                            running = false;
+                            cols_run = n;
+                        }
+                    }
+                    j += 8;
+                    if (!__any_sync(FULL, running)) break;
+                    jend = (int32_t)__reduce_min_sync(FULL, running ? (unsigned)n : 0x7FFFFFFFu);
+                    if (j < next_check) continue;
+                }
+                // the windows' minima; lanes predicted to be rejected within half as
+                // many columns again keep the task going
+                const int32_t lb = T + diag_min<W>(P, M, s_tab);
+                if (running && lb > K) {
+                    running = false;
+                    cols_run = j;
+                }
+                const unsigned left = __ballot_sync(FULL, running);
+                if (left == 0u) break;
+                const float rem = (float)(K + 1 - lb) * (float)j / (float)(lb > 1 ? lb : 1);
+                const bool soon = running && rem <= 0.5f * (float)j;
+                const unsigned far = __reduce_max_sync(FULL, soon ? (unsigned)rem + 1u : 0u);
+                if (far > 0u) {
+                    next_check = j + (int32_t)((far + 7u) & ~7u);
+                } else {
+                    const int32_t most = (int32_t)__reduce_max_sync(FULL, running ? (unsigned)(n - j) : 0u);
+                    if (vo.defer && __popc(left) <= SX_DEFER_MAX && most > j / 2) {
+                        // similar pairs: to the persistent verifier
+                        unsigned long long at = 0;
+                        if (lane == 0) at = atomicAdd(vo.defer_count, (unsigned long long)__popc(left));
+                        at = __shfl_sync(FULL, at, 0);
+                        if (running) {
+                            vo.defer[at + __popc(left & ((1u << lane) - 1u))] = pr;
+                            deferred = true;
+                            running = false;
+                            cols_run = j;
+                        }
+                        break;
+                    }
+                    next_check = j + 64;
+                }
+                jend = (int32_t)__reduce_min_sync(FULL, running ? (unsigned)n : 0x7FFFFFFFu);
             }
         }
-        if (valid && !rev) emit_result(vo, first + slot_pair, pairs, pass);
+        if (valid && !deferred) {
+            emit_result(vo, first + lane, pairs, pass);
+            loc_cells += band_cells(m, n, K);   // a deferred pair's are counted by its second verifier
+        }
         if (valid) {
-            if (!rev) loc_cells += band_cells(m, n, K);
             const int32_t d = m - n;   // the pair's own band: ((K - d) >> 1) + ((K + d) >> 1) + 1 diagonals
             loc_cols += (unsigned long long)cols_run * (unsigned long long)((((K - d) >> 1) + ((K + d) >> 1) + 64) >> 6);
         }
-        __syncwarp();   // the shared area is rebuilt by the next task
     }
     // work counters: one atomic per warp (per-pair atomics on two addresses
     // serialise in the memory system)
@@ -362,13 +328,13 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     }
 }
 
-// tcount[x] = tasks of string x (up to 16 of its pairs each); tcount[n] = 0.
+// tcount[x] = tasks of group x (up to SX_PAIRS of its pairs each); tcount[n] = 0.
 __global__ void sx_task_counts_kernel(const uint32_t *__restrict__ bins, int64_t n, uint32_t *__restrict__ tcount) {
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
-        tcount[x] = x < n ? (bins[x] + 15u) / 16u : 0u;
+        tcount[x] = x < n ? (bins[x] + SX_PAIRS - 1u) / SX_PAIRS : 0u;
 }
 
-// The tasks of string x: (first pair << 5) | pairs, over its run of candidates
+// The tasks of group x: (first pair << 6) | pairs, over its run of candidates
 // [ends[x] - bins[x], ends[x]).
 __global__ void sx_tasks_kernel(const uint32_t *__restrict__ bins, const uint64_t *__restrict__ ends, int64_t n,
                                 const uint64_t *__restrict__ tstart, uint64_t *__restrict__ tasks) {
@@ -376,59 +342,58 @@ __global__ void sx_tasks_kernel(const uint32_t *__restrict__ bins, const uint64_
         const uint32_t c = bins[x];
         if (!c) continue;
         const uint64_t base = ends[x] - c, t0 = tstart[x];
-        for (uint32_t k = 0; 16u * k < c; k++) {
-            const uint32_t left = c - 16u * k;
-            tasks[t0 + k] = ((base + 16ull * k) << 5) | (uint64_t)(left < 16u ? left : 16u);
+        for (uint32_t k = 0; k * SX_PAIRS < c; k++) {
+            const uint32_t left = c - k * SX_PAIRS;
+            tasks[t0 + k] = ((base + (uint64_t)k * SX_PAIRS) << 6) | (uint64_t)(left < SX_PAIRS ? left : SX_PAIRS);
         }
     }
 }
 
-template <int W1, int B>
+// Ring row stride: both copies of W + 1 words, odd (lanes reading different
+// symbols spread over the banks).
+int sx_row(int W) { return 2 * (W + 1) + 1; }
+
+template <int W, int B>
 cudaError_t launch_sx_t(const uint4 *packed, const uint64_t *pofs, const int32_t *lens, int64_t n, uint32_t alpha,
                         const uint64_t *pairs, const uint64_t *tasks, const unsigned long long *ntasks_dev,
                         int64_t ntasks_cap, int32_t K, VerifyOut vo, cudaStream_t s) {
-    const int RS = (W1 & 1) ? W1 : W1 + 1;   // odd: lanes reading different symbols spread over the banks
-    const size_t rings = 2 * (size_t)alpha * RS, dumpw = 32 * (size_t)(2 * W1 + 2);
-    const size_t warp_words = rings > dumpw ? rings : dumpw;
-    const size_t smem = warp_words * sizeof(uint64_t) * SX_WARPS;
+    const size_t smem = sx_smem_bytes(W, alpha);
     if (smem > 220 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(verify_sx_kernel<W1, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(verify_sx_kernel<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_sx_kernel<W1, B>, SX_WARPS * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_sx_kernel<W, B>, SX_WARPS * 32, smem);
     if (per_sm < 1) per_sm = 1;
     int64_t blocks = (int64_t)sms * per_sm;
     const int64_t need = (ntasks_cap + SX_WARPS - 1) / SX_WARPS;
     if (blocks > need) blocks = need > 0 ? need : 1;
-    verify_sx_kernel<W1, B><<<(unsigned)blocks, SX_WARPS * 32, smem, s>>>(
-        packed, pofs, lens, n, alpha, pairs, tasks, ntasks_dev, ntasks_cap, K, RS, (int32_t)warp_words, vo);
+    verify_sx_kernel<W, B><<<(unsigned)blocks, SX_WARPS * 32, smem, s>>>(
+        packed, pofs, lens, n, alpha, pairs, tasks, ntasks_dev, ntasks_cap, K, sx_row(W), (int32_t)(alpha * sx_row(W)),
+        vo);
     note_launches(1);
     return cudaGetLastError();
 }
 
 }  // namespace
 
+int sx_task_pairs() { return SX_PAIRS; }
+
 SxBand sx_band(int32_t K) {
-    const int words = (K + 1 + 63) / 64;   // ceil((K + 1) / 64)
-    int W = words, slack = 64 * words - (K + 1);
+    const int words = (K + 32) / 32;   // ceil((K + 1) / 32)
+    int W = words, slack = 32 * words - (K + 1);
     if (2 * slack + 1 < 7) {   // classes narrower than 7 would split the strings' pairs too finely
         W += 1;
-        slack += 64;
+        slack += 32;
     }
     uint32_t D = 2u * (uint32_t)slack + 1u;
     if (D > (uint32_t)K + 1u) D = (uint32_t)K + 1u;
-    return SxBand{W + 1, D, ((uint32_t)K + 1u + D - 1u) / D};
+    return SxBand{W, D, ((uint32_t)K + 1u + D - 1u) / D};
 }
 
-
-size_t sx_smem_bytes(int W1, uint32_t alpha) {
-    const size_t RS = (W1 & 1) ? W1 : W1 + 1;
-    const size_t rings = 2 * (size_t)alpha * RS, dumpw = 32 * (size_t)(2 * W1 + 2);
-    return (rings > dumpw ? rings : dumpw) * sizeof(uint64_t) * SX_WARPS;
-}
+size_t sx_smem_bytes(int W, uint32_t alpha) { return (size_t)alpha * sx_row(W) * sizeof(uint32_t) * SX_WARPS; }
 
 cudaError_t launch_sx_tasks(const uint32_t *bins, const uint64_t *ends, int64_t n, uint32_t *tcount, uint64_t *tstart,
                             unsigned long long *ntasks_dev, void *scan_tmp, uint64_t *tasks, cudaStream_t s) {
@@ -443,17 +408,17 @@ cudaError_t launch_sx_tasks(const uint32_t *bins, const uint64_t *ends, int64_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_verify_sx(int W1, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
+cudaError_t launch_verify_sx(int W, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
                              uint32_t alpha, const uint64_t *pairs, const uint64_t *tasks,
                              const unsigned long long *ntasks_dev, int64_t ntasks_cap, int32_t K, VerifyOut vo,
                              cudaStream_t s) {
     if (ntasks_cap == 0) return cudaGetLastError();
 #define EJ_SX(WW)                                                                                          \
-    if (W1 == WW) {                                                                                        \
+    if (W == WW) {                                                                                        \
         if (B == 2) return launch_sx_t<WW, 2>(packed, pofs, lens, n, alpha, pairs, tasks, ntasks_dev, ntasks_cap, K, vo, s); \
         return launch_sx_t<WW, 8>(packed, pofs, lens, n, alpha, pairs, tasks, ntasks_dev, ntasks_cap, K, vo, s);   \
     }
-    EJ_SX(2) EJ_SX(3) EJ_SX(4) EJ_SX(5) EJ_SX(6) EJ_SX(7) EJ_SX(8) EJ_SX(9) EJ_SX(10) EJ_SX(11) EJ_SX(12)
+    EJ_SX(1) EJ_SX(2) EJ_SX(3) EJ_SX(4) EJ_SX(5) EJ_SX(6) EJ_SX(7) EJ_SX(8) EJ_SX(9) EJ_SX(10) EJ_SX(11) EJ_SX(12)
 #undef EJ_SX
     return cudaErrorInvalidValue;
 }
