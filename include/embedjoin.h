@@ -378,7 +378,8 @@ void ej_batch_destroy(ej_batch *batch);
  *   buckets: 0 (default) or 1: equal signatures are grouped by hashing (per
  *     table an open-addressing set whose slots head lists of records); a
  *     record pairs with the later records of its list, so a bucket of b strings
- *     costs b*(b-1)/2 length checks. In a batch, 0 also shares buckets: joins
+ *     costs b*(b-1)/2 length checks. The shared-string verifier's candidates come
+ *     from sorted tables whatever is chosen here. In a batch, 0 also shares buckets: joins
  *     with the same seed, L, r and m (up to 4) take their pairs from the
  *     buckets of the one with the smallest z, whose signatures are the coarsest
  *     (a signature of z samples is one of more samples modulo (|alphabet|+1)^z),

@@ -31,9 +31,8 @@ enum BufId {
     B_HASH, B_APP, B_JCOUNT, B_NEXT, B_HCOUNT, B_BINS, B_TICKETS, B_BKEYS, B_BHEADS, B_BNEXT, B_FBINS, B_FSTARTS,
     B_FSCAN,
     B_PLUS_SUBLEN, B_PLUS_WHOLE, B_PLUS_SUBOFF, B_PLUS_BYTES, B_PLUS_SCAN, B_PLUS_CAND,
-    B_SX_TCOUNT, B_SX_TSTART, B_SX_TASKS, B_SX_SCAN,
+    B_SX_TASKS, B_GREC, B_GPOS, B_GFP,
     B_GROUP_IDX, B_GROUP_OFF, B_GROUP_BYTES, B_GROUP_OUT,
-    B_DG_TEMP, B_GSTART,
     B_NUM
 };
 
@@ -691,7 +690,8 @@ int verify_dev(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *
 struct BackState {
     bool hashed = false;
     bool table_smem = false;           // hashed, each table's buckets built in shared memory
-    const uint64_t *keys = nullptr;    // the signatures (table_smem)
+    bool grouped = false;              // sorted tables feeding the shared-string verifier's tasks (ej_group.cu)
+    const uint64_t *keys = nullptr;    // the signatures (table_smem, grouped)
     const uint64_t *srk = nullptr;
     const uint32_t *srid = nullptr;
     uint32_t *bnext = nullptr;
@@ -707,13 +707,36 @@ constexpr unsigned SMEM_BUCKET_MAX = 256;
 // tables with length windows instead of hashed buckets.
 constexpr unsigned SORTED_BUCKET_MIN = 4096;
 
+// Threads per block of the persistent verifier this join uses, 0 for the
+// grid-strided one. Mode 0 picks the persistent verifier for long strings only
+// (mean length >= 2048): on short, mostly rejected pairs its per-pair refill
+// costs more than it saves (measured 2x slower on the protein-like shape).
+int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
+    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
+    const bool want_pq = ctx->sched.mode == 1 || (ctx->sched.mode == 0 && long_pairs);
+    return (vc.G == 2 && want_pq) ? pq_threads_for(pq_words(p->K), p->alphabet_size) : 0;
+}
+
+// The shared-string verifier (mode 3; mode 0 for short strings over more than
+// four symbols, whose per-lane match-mask rings would leave the other verifiers
+// a few warps per SM): the band within SX_MAX_WORDS words, the warps' rings within
+// the block's budget.
+bool sx_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
+    const int W = sx_band(p->K).W;
+    if (vc.G != 2 || W > SX_MAX_WORDS || sx_smem_bytes(W, p->alphabet_size) > 220 * 1024) return false;
+    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
+    return ctx->sched.mode == 3 || (ctx->sched.mode == 0 && !long_pairs && p->alphabet_size > 4);
+}
+
 int back_buckets(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *keys, BackState *bs,
                  cudaStream_t s) {
     const int64_t n = pl.st.n, T = (int64_t)p->r * p->m;
     uint32_t *derr = nullptr;
     CKS(ensure_t(ctx, B_DERR, 8, &derr));
     CK(cudaMemsetAsync(derr, 0, 4, s));
-    bs->hashed = ctx->sched.buckets != 2 && n * T < (int64_t)0xFFFFFFFFll;
+    CKS(pick_verify(ctx, p, pl, &bs->vc));
+    bs->grouped = sx_choice(ctx, pl, p, bs->vc);
+    bs->hashed = !bs->grouped && ctx->sched.buckets != 2 && n * T < (int64_t)0xFFFFFFFFll;
     bs->table_smem = bs->hashed && bucket_table_smem(n) > 0 && !ctx->no_smem_buckets;
     bs->keys = keys;
     if (bs->table_smem) {
@@ -732,7 +755,6 @@ int back_buckets(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t
     } else {
         CKS(sorted_records(ctx, pl, p, keys, &bs->srk, &bs->srid, s));
     }
-    CKS(pick_verify(ctx, p, pl, &bs->vc));
     return EJ_OK;
 }
 
@@ -740,25 +762,16 @@ uint64_t raw_cap_start(ej_ctx *ctx, int64_t n) {
     return ctx->raw_cap_hint ? ctx->raw_cap_hint : (uint64_t)(n * 4 > 65536 ? n * 4 : 65536);
 }
 
-// Threads per block of the persistent verifier this join uses, 0 for the
-// grid-strided one. Mode 0 picks the persistent verifier for long strings only
-// (mean length >= 2048): on short, mostly rejected pairs its per-pair refill
-// costs more than it saves (measured 2x slower on the protein-like shape).
-int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
-    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
-    const bool want_pq = ctx->sched.mode == 1 || (ctx->sched.mode == 0 && long_pairs);
-    return (vc.G == 2 && want_pq) ? pq_threads_for(pq_words(p->K), p->alphabet_size) : 0;
+// Pair slots of the buffers of an attempt with capacity cap: the raw pairs, or
+// the whole tasks of the shared-string verifier.
+uint64_t back_slots(const Plan &pl, const ej_params *p, const BackState &bs, uint64_t cap) {
+    return bs.grouped ? 32 * (uint64_t)group_task_cap(cap, pl.st.n, sx_band(p->K).nclass) : cap;
 }
 
-// The shared-string verifier (mode 3; mode 0 for short strings over more than
-// four symbols, where the per-lane match-mask rings of the grid-strided
-// verifier leave one or two warps per SM): two lanes per pair, the band within
-// 12 words per lane, the warp's shared area within the block's budget.
-bool sx_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
-    const int W = sx_band(p->K).W;
-    if (vc.G != 2 || W > SX_MAX_WORDS || sx_smem_bytes(W, p->alphabet_size) > 220 * 1024) return false;
-    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
-    return ctx->sched.mode == 3 || (ctx->sched.mode == 0 && !long_pairs && p->alphabet_size > 4);
+// The capacity an attempt whose counters are hc would have needed; 0 if it fits.
+uint64_t back_needs(const Plan &pl, const ej_params *p, const BackState &bs, const unsigned long long hc[8], uint64_t cap) {
+    if (!bs.grouped) return hc[0] > cap ? hc[0] : 0;
+    return 32 * hc[7] > back_slots(pl, p, bs, cap) ? 32 * hc[7] : 0;
 }
 
 // verify_after / verify_done (optional): the verifier launch waits for the
@@ -774,23 +787,37 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     uint32_t *derr = (uint32_t *)ctx->bufs[B_DERR].p;
     uint64_t hsize = 1;
     while (hsize < 2 * cap) hsize <<= 1;
-    uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr, *spare = nullptr;
-    CKS(ensure_t(ctx, B_RAW, (size_t)cap, &raw));
-    CKS(ensure_t(ctx, B_CAND, (size_t)cap, &cand));
-    CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
+    const uint64_t slots = back_slots(pl, p, bs, cap);
+    uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr;
+    CKS(ensure_t(ctx, B_RAW, (size_t)slots, &raw));
+    CKS(ensure_t(ctx, B_CAND, (size_t)slots, &cand));
+    CKS(ensure_t(ctx, B_APP, (size_t)slots, &app));
     // the verifier and the candidate order it takes
-    const bool sx = !defer && sx_choice(ctx, pl, p, bs.vc);
+    const bool sx = bs.grouped;
     const int pq_threads = sx ? 0 : pq_choice(ctx, pl, p, bs.vc);
-    // the shared-string verifier needs its pairs grouped by their longer string
-    const int order = sx ? 5 : bs.any_order ? 2 : ctx->sched.order != 0 ? ctx->sched.order : (pq_threads > 0 ? 4 : 3);
+    const int order = bs.any_order ? 2 : ctx->sched.order != 0 ? ctx->sched.order : (pq_threads > 0 ? 4 : 3);
+    const SxBand sb = sx ? sx_band(p->K) : SxBand{0, 1u, 1u};
+    uint32_t *tasks = nullptr;   // the shared-string verifier's tasks: pairs of each, 32 slots of cand
     // emitted: the raw pairs and counters [0], [1] are already written (shared
     // buckets of a batch)
     CK(cudaMemsetAsync(emitted ? cnt + 2 : cnt, 0, (emitted ? JCOUNT_LEN - 2 : JCOUNT_LEN) * sizeof(unsigned long long), s));
-    if (!sx) {   // the shared-string verifier's candidates are deduplicated by sorting
+    if (!sx) {   // the shared-string verifier's candidates are distinct when they are emitted
         CKS(ensure_t(ctx, B_HASH, (size_t)hsize, &table));
         CK(cudaMemsetAsync(table, 0xFF, hsize * sizeof(uint64_t), s));
     }
     if (emitted) {
+    } else if (sx) {
+        // distinct candidates in the shared-string verifier's tasks, from the sorted tables
+        uint64_t *rec = nullptr;
+        uint32_t *pos = nullptr;
+        void *fp = nullptr;
+        CKS(ensure_t(ctx, B_GREC, (size_t)(n * T), &rec));
+        CKS(ensure_t(ctx, B_GPOS, (size_t)(n * T), &pos));
+        CKS(ensure(ctx, B_GFP, fingerprint_bytes(n, T), &fp));
+        CKS(ensure_t(ctx, B_SX_TASKS, (size_t)(slots / 32), &tasks));
+        CK(launch_group_prep(bs.srk, bs.srid, bs.keys, pl.lens, n, T, rec, pos, (uint4 *)fp, cnt, s));
+        CK(launch_group_emit(bs.srk, rec, pos, bs.keys, (const uint4 *)fp, pl.lens, n, T, p->K, sb.width, sb.nclass,
+                             (int64_t)(slots / 32), cand, tasks, cnt, s));
     } else if (bs.table_smem) {
         SharedEmit se{};
         se.njoins = 1;
@@ -810,21 +837,8 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     // protein-like / text-like shapes
     uint32_t *fbins = nullptr;
     uint64_t *fstarts = nullptr;
-    // the shared-string verifier's window and length-difference classes
-    const SxBand sb = sx ? sx_band(p->K) : SxBand{0, 1u, 1u};
-    const int64_t nb = n * (int64_t)sb.nclass;   // the shared-string verifier's candidate groups
     if (sx) {
-        // the shared-string verifier's tasks: the distinct pairs sorted by their
-        // longer string and the class of their length difference
-        void *dgt = nullptr;
-        uint64_t *gstart = nullptr, *sorted_cand = nullptr;
-        CKS(ensure_t(ctx, B_FBINS, (size_t)nb + 1, &fbins));
-        CKS(ensure_t(ctx, B_FSTARTS, (size_t)nb + 2, &fstarts));
-        CKS(ensure_t(ctx, B_GSTART, (size_t)nb + 1, &gstart));
-        CKS(ensure(ctx, B_DG_TEMP, dedup_grouped_temp_bytes(cap), &dgt));
-        CK(launch_dedup_grouped(raw, cand, cap, n, pl.lens, sb.nclass, sb.width, cnt, dgt, fbins, fstarts, gstart,
-                                &sorted_cand, &spare, s));
-        cand = sorted_cand;
+        // distinct and in order already
     } else if (order == 3 || order == 5) {
         // candidates ordered by their first string (a warp's pairs share it), or
         // by their longer string
@@ -855,44 +869,33 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     }
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[3], s));
     if (defer) {
-        *defer = VerifySeg{cand, cnt + 2, cap, p->K, app, cnt + 3, cap, cnt + 4, derr};
+        *defer = VerifySeg{cand, cnt + 2, cap, p->K, app, cnt + 3, cap, cnt + 4, derr};   // (never grouped)
         return EJ_OK;
     }
     unsigned int *tickets = nullptr;
     CKS(ensure_t(ctx, B_TICKETS, (size_t)SM_TICKETS, &tickets));
     CK(cudaMemsetAsync(tickets, 0, SM_TICKETS * sizeof(unsigned int), s));
-    VerifyOut vo{nullptr, app, cnt + 3, cap, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
+    VerifyOut vo{nullptr, app, cnt + 3, slots, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
     vo.max_passes = ctx->loop_bound;
     const VerifyConfig &vc = bs.vc;
     if (sx) {
-        // warp tasks of candidates sharing their longer string and the class of
-        // their length difference
-        const int64_t tcap = (int64_t)(cap / (uint64_t)sx_task_pairs()) + nb + 1;
-        uint32_t *tcount = nullptr;
-        uint64_t *tstart = nullptr, *tasks = nullptr;
-        void *tscan = nullptr;
-        CKS(ensure_t(ctx, B_SX_TCOUNT, (size_t)nb + 1, &tcount));
-        CKS(ensure_t(ctx, B_SX_TSTART, (size_t)nb + 1, &tstart));
-        CKS(ensure_t(ctx, B_SX_TASKS, (size_t)tcap, &tasks));
-        CKS(ensure(ctx, B_SX_SCAN, scan_temp_bytes(nb + 1), &tscan));
-        CK(launch_sx_tasks(fbins, fstarts, nb, tcount, tstart, cnt + 7, tscan, tasks, s));
         if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));
         // pairs that outlive the rest of their task (similar strings) go to the
         // persistent verifier, where that has a block size for them
         const int pq_after = pq_threads_for(pq_words(p->K), p->alphabet_size);
         if (pq_after > 0) {
-            vo.defer = spare;
+            vo.defer = raw;
             vo.defer_count = cnt + 8;
         }
         CK(launch_verify_sx(sb.W, pl.packed, pl.pofs, pl.B, pl.lens, n, p->alphabet_size, cand, tasks, cnt + 7,
-                            tcap, p->K, vo, s));
+                            (int64_t)(slots / 32), p->K, vo, s));
         if (pq_after > 0) {
             VerifyOut v2 = vo;
             v2.defer = nullptr;
             v2.np_dev = cnt + 8;
             CK(launch_verify_pq(pq_words(p->K), pq_after, ctx->sched.slots_per_warp ? ctx->sched.slots_per_warp : 16,
                                 ctx->sched.warps_per_subpartition, pl.packed, pl.pofs, pl.B, pl.lens, n,
-                                p->alphabet_size, spare, (int64_t)cap, p->K, v2, s));
+                                p->alphabet_size, raw, (int64_t)slots, p->K, v2, s));
         }
     } else {
     if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));
@@ -925,9 +928,9 @@ int back_segment(ej_ctx *ctx, const ej_params *p, uint64_t cap, VerifySeg *seg) 
 }
 
 // Counters of the last attempt: [0] raw, [1] max bucket, [2] candidates,
-// [3] output, [4] band cells, [5] word columns, [6] device error bits.
+// [3] output, [4] band cells, [5] word columns, [6] device error bits, [7] tasks.
 int back_read(ej_ctx *ctx, unsigned long long hc[8], cudaStream_t s) {
-    CK(cudaMemcpyAsync(ctx->h_cnt, ctx->bufs[B_JCOUNT].p, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(ctx->h_cnt, ctx->bufs[B_JCOUNT].p, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(ctx->h_cnt + 6, ctx->bufs[B_DERR].p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     memcpy(hc, ctx->h_cnt, 8 * sizeof(unsigned long long));
@@ -991,9 +994,10 @@ int join_back(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *k
     for (int attempt = 0;; attempt++) {
         CKS(back_attempt(ctx, pl, p, bs, cap, s));
         CKS(back_read(ctx, hc, s));
-        if (hc[0] <= cap) break;
+        const uint64_t need = back_needs(pl, p, bs, hc, cap);
+        if (!need) break;
         if (attempt > 0) return fail(ctx, EJ_ERR_CUDA, "raw pair count changed between attempts");
-        cap = hc[0] + hc[0] / 4 + 1024;
+        cap = need + need / 4 + 1024;
     }
     ctx->raw_cap_hint = cap;
     return back_finish(ctx, pl, p, hc, out, capacity, n_out, stats, s);
@@ -1136,11 +1140,13 @@ int tune_join(ej_ctx *ctx, const Plan &pl, const ej_params *p, uint64_t *keys, c
     for (int attempt = 0;; attempt++) {
         CKS(back_attempt(ctx, pl, p, bs, cap, s));
         CKS(back_read(ctx, hc, s));
-        if (hc[0] <= cap) break;
+        const uint64_t need = back_needs(pl, p, bs, hc, cap);
+        if (!need) break;
         if (attempt > 0) return fail(ctx, EJ_ERR_CUDA, "raw pair count changed between attempts");
-        cap = hc[0] + hc[0] / 4 + 1024;
+        cap = need + need / 4 + 1024;
     }
     ctx->raw_cap_hint = cap;
+    cap = std::max<uint64_t>(cap, hc[0] + hc[0] / 4 + 1024);   // every choice's raw pairs fit
     return tune_back(ctx, pl, p, keys, cap, s, out);
 }
 
@@ -1180,7 +1186,7 @@ struct BatchJoin {
     uint64_t modulus = 0;             // keys = src keys mod modulus (0: same z)
     bool alias = false;               // same r, m, z as src: read src's keys directly
     bool in_walk = false;             // same r, m, smaller z: written by src's walk kernel
-    uint64_t ncand = 0;               // candidates in the eager pass
+    uint64_t ncand = 0, nraw = 0;     // candidates and raw pairs in the eager pass
     int seg = -1;                     // share of the merged verifier launch (-1: none)
     int bucket_owner = -1;            // join whose buckets give this join's pairs (-1: its own)
     std::vector<int> bucket_members;  // owner: the joins (itself first) its buckets serve
@@ -2399,19 +2405,19 @@ int ej_batch_create(ej_ctx *ctx, const ej_strings *S, const ej_params *params, i
         if (j.src < 0 && (st = batch_join_keys(b->joins, j, s)) != EJ_OK) return bail(st);
     for (auto &j : b->joins)
         if (j.src >= 0 && (st = batch_join_keys(b->joins, j, s)) != EJ_OK) return bail(st);
-    for (auto &j : b->joins) {
-        if ((st = back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s)) != EJ_OK) return bail(st);
+    auto size_join = [&](BatchJoin &j) -> int {
+        CKS(back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s));
         uint64_t cap = raw_cap_start(j.sub, b->pl.st.n);
         unsigned long long hc[8];
         for (int attempt = 0;; attempt++) {
-            if ((st = back_attempt(j.sub, j.pl, &j.p, j.bs, cap, s)) != EJ_OK) return bail(st);
-            if ((st = back_read(j.sub, hc, s)) != EJ_OK) return bail(st);
+            CKS(back_attempt(j.sub, j.pl, &j.p, j.bs, cap, s));
+            CKS(back_read(j.sub, hc, s));
             if (j.bs.hashed && ctx->sched.buckets == 0 && hc[1] > (unsigned long long)SORTED_BUCKET_MIN) {
                 // buckets of thousands of records: a list walks all b(b-1)/2 pairs
                 // of a bucket, the sorted tables only the pairs within the length
                 // window (measured 2x faster on the protein-like shape)
                 j.sub->sched.buckets = 2;
-                if ((st = back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s)) != EJ_OK) return bail(st);
+                CKS(back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s));
                 attempt = -1;
                 continue;
             }
@@ -2420,20 +2426,29 @@ int ej_batch_create(ej_ctx *ctx, const ej_strings *S, const ej_params *params, i
                 // in b(b-1)/2 steps on one SM: huge buckets go to global memory,
                 // where every SM takes part
                 j.sub->no_smem_buckets = true;
-                if ((st = back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s)) != EJ_OK) return bail(st);
+                CKS(back_buckets(j.sub, j.pl, &j.p, j.keys, &j.bs, s));
                 attempt = -1;
                 continue;
             }
-            if (hc[0] <= cap) break;
-            if (attempt > 2) return bail(fail(ctx, EJ_ERR_CUDA, "raw pair count changed between attempts"));
-            cap = hc[0] + hc[0] / 4 + 1024;
+            const uint64_t need = back_needs(j.pl, &j.p, j.bs, hc, cap);
+            if (!need) break;
+            if (attempt > 2) return fail(ctx, EJ_ERR_CUDA, "raw pair count changed between attempts");
+            cap = need + need / 4 + 1024;
         }
         j.ncand = hc[2];
+        j.nraw = hc[0];
         j.cap = cap + cap / 8 + 1024;
-        if ((st = back_attempt(j.sub, j.pl, &j.p, j.bs, j.cap, s)) != EJ_OK) return bail(st);
+        return back_attempt(j.sub, j.pl, &j.p, j.bs, j.cap, s);
+    };
+    for (auto &j : b->joins) {
+        if ((st = size_join(j)) != EJ_OK) return bail(st);
         if (flags & EJ_BATCH_AUTOTUNE) {
+            // the choices are timed at a capacity that all raw pairs fit; the chosen
+            // one is sized anew (its buckets may be others)
+            j.cap = std::max<uint64_t>(j.cap, j.nraw + j.nraw / 8 + 1024);
             float ms = 0.f;
             if ((st = batch_autotune(ctx, j, s, &ms)) != EJ_OK) return bail(st);
+            if ((st = size_join(j)) != EJ_OK) return bail(st);
         }
         if (cudaStreamSynchronize(s) != cudaSuccess) return bail(fail(ctx, EJ_ERR_CUDA, "eager pass failed"));
     }
@@ -2549,12 +2564,12 @@ int ej_batch_result(ej_batch *b, int32_t i, uint64_t *out, int64_t capacity, int
     unsigned long long hc[8];
     memcpy(hc, b->h_stat + 16 * (size_t)i, 6 * sizeof(unsigned long long));
     hc[6] = b->h_stat[16 * (size_t)i + 8] & 0xffffffffull;
-    hc[7] = 0;
+    hc[7] = b->h_stat[16 * (size_t)i + 7];
     if ((uint32_t)hc[6] & DERR_PAIR) return fail(ctx, EJ_ERR_INVALID_ARG, "internal: pair index out of range");
     if ((uint32_t)hc[6] & DERR_TIMEOUT)
         return fail(ctx, EJ_ERR_TIMEOUT, "the persistent verifier gave up after its bound of loop passes per warp");
     if ((uint32_t)hc[6] & DERR_GUARD) return fail(ctx, EJ_ERR_CUDA, "internal: a work bound was exceeded");
-    if (hc[0] > j.cap)
+    if (back_needs(j.pl, &j.p, j.bs, hc, j.cap))
         return fail(ctx, EJ_ERR_CAPACITY, "raw pairs (%llu) exceed the batch's capacity (%llu): re-create the batch",
                     hc[0], (unsigned long long)j.cap);
     int64_t cnt = 0;

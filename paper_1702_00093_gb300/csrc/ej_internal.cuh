@@ -280,18 +280,6 @@ cudaError_t launch_dedup(const uint64_t *raw, uint64_t cap, uint64_t *table, uin
 // max_len to 256 classes). hcount (hsize uint32) and bins (count_bins() uint64)
 // start at zero.
 int count_bins();
-// Dedup by sorting, for the shared-string verifier: raw[0 .. counters[0]) (the
-// rest of cap is not read) is sorted by (longer string, class of the length
-// difference, other string) with the LSD radix sort (alt: cap entries), the
-// distinct pairs written in that order to *cand_out (raw or alt; *free_out is the
-// other, cap entries that hold nothing any more) and counted in counters[2]; per group g = x * nclass
-// + class: bins[g] (nb + 1 uint32, cleared here) its count, ends[g] its end
-// offset (nb uint64), gstart (nb uint64) scratch. temp: dedup_grouped_temp_bytes.
-size_t dedup_grouped_temp_bytes(uint64_t cap);
-cudaError_t launch_dedup_grouped(uint64_t *raw, uint64_t *alt, uint64_t cap, int64_t n, const int32_t *lens,
-                                 uint32_t nclass, uint32_t width, unsigned long long *counters, void *temp,
-                                 uint32_t *bins, uint64_t *ends, uint64_t *gstart, uint64_t **cand_out,
-                                 uint64_t **free_out, cudaStream_t s);
 struct VerifySeg;
 // Union of the candidate lists of a merged launch's joins (segs[0 .. nseg)):
 // every distinct pair once in upairs, with the mask of the joins that list it
@@ -348,11 +336,23 @@ cudaError_t launch_dedup_by_first(const uint64_t *raw, uint64_t cap, uint64_t *t
                                   int64_t n, uint32_t *bins, uint64_t *starts, void *scan_tmp, uint64_t *cand,
                                   unsigned long long *counters, cudaStream_t s,
                                   const int32_t *longer_lens = nullptr);
-// Shared-string verifier (ej_verify_sx.cu): warp tasks of up to sx_task_pairs()
-// candidates that share their longer string and length-difference class, from
-// the groups of launch_dedup_grouped (nb groups; tcount nb+1 uint32, tstart nb+1
-// uint64, tasks up to candidates/sx_task_pairs() + nb entries; *ntasks_dev =
-// their number), and the verifier.
+// Candidates for the shared-string verifier (ej_group.cu). Task i is tasks[i] <= 32
+// pairs at pairs[32 i ..], all with the same longer string (the later one of two
+// equally long) and length-difference class; counters: [0] raw pairs, [1] largest
+// bucket, [2] candidates, [7] task numbers in use (beyond tcap nothing is
+// written). group_task_cap: the tasks that cap pairs may need. rk / rid: the
+// tables' records sorted by (signature, length, id); rec, pos: n T entries; fp:
+// fingerprint_bytes(n, T).
+int64_t group_task_cap(uint64_t cap, int64_t n, uint32_t nclass);
+size_t fingerprint_bytes(int64_t n, int64_t T);
+cudaError_t launch_group_prep(const uint64_t *rk, const uint32_t *rid, const uint64_t *keys, const int32_t *lens,
+                              int64_t n, int64_t T, uint64_t *rec, uint32_t *pos, uint4 *fp,
+                              unsigned long long *counters, cudaStream_t s);
+cudaError_t launch_group_emit(const uint64_t *rk, const uint64_t *rec, const uint32_t *pos, const uint64_t *keys,
+                              const uint4 *fp, const int32_t *lens, int64_t n, int64_t T, int32_t K, uint32_t width,
+                              uint32_t nclass, int64_t tcap, uint64_t *pairs, uint32_t *tasks,
+                              unsigned long long *counters, cudaStream_t s);
+// Shared-string verifier (ej_verify_sx.cu).
 // sx_band(K): the verifier's window of W 32-bit words and the class width and
 // count that keep a task's band within it: a task's length differences lie in
 // one class of width D, so its band (the diagonals a cost-K alignment of any of
@@ -364,10 +364,7 @@ struct SxBand {
 };
 constexpr int SX_MAX_WORDS = 12;
 SxBand sx_band(int32_t K);
-int sx_task_pairs();
 size_t sx_smem_bytes(int W, uint32_t alpha);
-cudaError_t launch_sx_tasks(const uint32_t *bins, const uint64_t *ends, int64_t n, uint32_t *tcount, uint64_t *tstart,
-                            unsigned long long *ntasks_dev, void *scan_tmp, uint64_t *tasks, cudaStream_t s);
 int small_sort_max();
 cudaError_t launch_small_sort(uint64_t *a, const unsigned long long *count_dev, uint64_t n_cap, cudaStream_t s);
 
@@ -475,11 +472,9 @@ int pq_threads_for(int W, uint32_t alpha);   // 0 if no block size fits
 cudaError_t launch_verify_pq(int W, int threads, int spw_force, int wps, const uint4 *packed, const uint64_t *pofs, int B,
                              const int32_t *lens, int64_t n, uint32_t alpha, const uint64_t *pairs, int64_t np,
                              int32_t K, VerifyOut vo, cudaStream_t s);
-// Shared-string verifier (W = 1..SX_MAX_WORDS): the pairs of tasks[0 .. *ntasks_dev)
-// (at most ntasks_cap), each task up to sx_task_pairs() pairs sharing their longer
-// string.
+// W = 1..SX_MAX_WORDS: the tasks 0 .. *ntasks_dev (at most ntasks_cap).
 cudaError_t launch_verify_sx(int W, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
-                             uint32_t alpha, const uint64_t *pairs, const uint64_t *tasks,
+                             uint32_t alpha, const uint64_t *pairs, const uint32_t *tasks,
                              const unsigned long long *ntasks_dev, int64_t ntasks_cap, int32_t K, VerifyOut vo,
                              cudaStream_t s);
 

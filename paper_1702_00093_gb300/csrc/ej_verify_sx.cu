@@ -43,7 +43,7 @@ namespace ej {
 namespace {
 
 constexpr int SX_WARPS = 4;       // warps per block
-constexpr int SX_PAIRS = 32;      // pairs per task
+constexpr int SX_PAIRS = 32;      // slots per task
 constexpr int SX_DEFER_MAX = 8;   // lanes left when a task hands its similar pairs over
 
 // Symbol i (0 <= i < m) of a packed string.
@@ -90,7 +90,7 @@ template <int W, int B>
 __global__ void __launch_bounds__(SX_WARPS * 32, sx_blocks<W>())
 verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ pofs,
                  const int32_t *__restrict__ lens, int64_t n_str, uint32_t alpha,
-                 const uint64_t *__restrict__ pairs, const uint64_t *__restrict__ tasks,
+                 const uint64_t *__restrict__ pairs, const uint32_t *__restrict__ tasks,
                  const unsigned long long *__restrict__ ntasks_dev, int64_t ntasks_cap, int32_t K, int32_t RS,
                  int32_t warp_words, VerifyOut vo) {
     uint32_t *__restrict__ err = vo.err;
@@ -103,28 +103,27 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     uint32_t *ring = sx_smem + (size_t)wib * warp_words;
-    const int64_t cap_t = (int64_t)*ntasks_dev;
-    const int64_t ntasks = cap_t < ntasks_cap ? cap_t : ntasks_cap;
+    const int64_t ntasks = (int64_t)*ntasks_dev;
+    if (ntasks > ntasks_cap) return;   // tasks are missing: the call is repeated with room for them
     const int64_t nw = (int64_t)gridDim.x * SX_WARPS;
     const int planes = alpha <= 1 ? 1 : 32 - __clz(alpha - 1u);
 
     unsigned long long loc_cells = 0, loc_cols = 0;
-    // a task's descriptor and this lane's pair are loaded during the task before
+    // a task's count and this lane's pair are loaded during the task before
     int64_t t = (int64_t)blockIdx.x * SX_WARPS + wib;
-    uint64_t tk_next = 0, pr_next = 0;
+    int cnt_next = 0;
+    uint64_t pr_next = 0;
     if (t < ntasks) {
-        tk_next = tasks[t];
-        if (lane < (int)(tk_next & 63u)) pr_next = pairs[(int64_t)(tk_next >> 6) + lane];
+        cnt_next = (int)tasks[t];
+        if (lane < cnt_next) pr_next = pairs[t * SX_PAIRS + lane];
     }
     for (; t < ntasks; t += nw) {   // warp-uniform
-        const uint64_t tk = tk_next;
         const uint64_t pr = pr_next;
+        bool valid = lane < cnt_next;
         if (t + nw < ntasks) {
-            tk_next = tasks[t + nw];
-            if (lane < (int)(tk_next & 63u)) pr_next = pairs[(int64_t)(tk_next >> 6) + lane];
+            cnt_next = (int)tasks[t + nw];
+            if (lane < cnt_next) pr_next = pairs[(t + nw) * SX_PAIRS + lane];
         }
-        const int64_t first = (int64_t)(tk >> 6);
-        bool valid = lane < (int)(tk & 63u);
         int64_t a = 0, b = 0;
         if (valid) {
             a = (int64_t)(pr >> 32);
@@ -135,7 +134,7 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             }
         }
         const int32_t la = valid ? lens[a] : 0, lb = valid ? lens[b] : 0;
-        const bool a_long = la >= lb;
+        const bool a_long = la > lb;   // of two equally long ones x is the later (a < b)
         const int64_t xi = a_long ? a : b, yi = a_long ? b : a;
         const int32_t m = a_long ? la : lb, n = a_long ? lb : la;
         // every pair of a task has the same x (its first pair's)
@@ -305,7 +304,7 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             }
         }
         if (valid && !deferred) {
-            emit_result(vo, first + lane, pairs, pass);
+            emit_result(vo, t * SX_PAIRS + lane, pairs, pass);
             loc_cells += band_cells(m, n, K);   // a deferred pair's are counted by its second verifier
         }
         if (valid) {
@@ -328,34 +327,13 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     }
 }
 
-// tcount[x] = tasks of group x (up to SX_PAIRS of its pairs each); tcount[n] = 0.
-__global__ void sx_task_counts_kernel(const uint32_t *__restrict__ bins, int64_t n, uint32_t *__restrict__ tcount) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
-        tcount[x] = x < n ? (bins[x] + SX_PAIRS - 1u) / SX_PAIRS : 0u;
-}
-
-// The tasks of group x: (first pair << 6) | pairs, over its run of candidates
-// [ends[x] - bins[x], ends[x]).
-__global__ void sx_tasks_kernel(const uint32_t *__restrict__ bins, const uint64_t *__restrict__ ends, int64_t n,
-                                const uint64_t *__restrict__ tstart, uint64_t *__restrict__ tasks) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t c = bins[x];
-        if (!c) continue;
-        const uint64_t base = ends[x] - c, t0 = tstart[x];
-        for (uint32_t k = 0; k * SX_PAIRS < c; k++) {
-            const uint32_t left = c - k * SX_PAIRS;
-            tasks[t0 + k] = ((base + (uint64_t)k * SX_PAIRS) << 6) | (uint64_t)(left < SX_PAIRS ? left : SX_PAIRS);
-        }
-    }
-}
-
 // Ring row stride: both copies of W + 1 words, odd (lanes reading different
 // symbols spread over the banks).
 int sx_row(int W) { return 2 * (W + 1) + 1; }
 
 template <int W, int B>
 cudaError_t launch_sx_t(const uint4 *packed, const uint64_t *pofs, const int32_t *lens, int64_t n, uint32_t alpha,
-                        const uint64_t *pairs, const uint64_t *tasks, const unsigned long long *ntasks_dev,
+                        const uint64_t *pairs, const uint32_t *tasks, const unsigned long long *ntasks_dev,
                         int64_t ntasks_cap, int32_t K, VerifyOut vo, cudaStream_t s) {
     const size_t smem = sx_smem_bytes(W, alpha);
     if (smem > 220 * 1024) return cudaErrorInvalidValue;
@@ -379,8 +357,6 @@ cudaError_t launch_sx_t(const uint4 *packed, const uint64_t *pofs, const int32_t
 
 }  // namespace
 
-int sx_task_pairs() { return SX_PAIRS; }
-
 SxBand sx_band(int32_t K) {
     const int words = (K + 32) / 32;   // ceil((K + 1) / 32)
     int W = words, slack = 32 * words - (K + 1);
@@ -395,21 +371,8 @@ SxBand sx_band(int32_t K) {
 
 size_t sx_smem_bytes(int W, uint32_t alpha) { return (size_t)alpha * sx_row(W) * sizeof(uint32_t) * SX_WARPS; }
 
-cudaError_t launch_sx_tasks(const uint32_t *bins, const uint64_t *ends, int64_t n, uint32_t *tcount, uint64_t *tstart,
-                            unsigned long long *ntasks_dev, void *scan_tmp, uint64_t *tasks, cudaStream_t s) {
-    int64_t g = (n + 256) / 256;
-    const unsigned gs = (unsigned)(g > 4096 ? 4096 : (g ? g : 1));
-    sx_task_counts_kernel<<<gs, 256, 0, s>>>(bins, n, tcount);
-    note_launches(1);
-    cudaError_t e = exclusive_scan_u32(tcount, tstart, n + 1, (uint64_t *)ntasks_dev, scan_tmp, s);
-    if (e != cudaSuccess) return e;
-    sx_tasks_kernel<<<gs, 256, 0, s>>>(bins, ends, n, tstart, tasks);
-    note_launches(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_verify_sx(int W, const uint4 *packed, const uint64_t *pofs, int B, const int32_t *lens, int64_t n,
-                             uint32_t alpha, const uint64_t *pairs, const uint64_t *tasks,
+                             uint32_t alpha, const uint64_t *pairs, const uint32_t *tasks,
                              const unsigned long long *ntasks_dev, int64_t ntasks_cap, int32_t K, VerifyOut vo,
                              cudaStream_t s) {
     if (ntasks_cap == 0) return cudaGetLastError();
