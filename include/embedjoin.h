@@ -345,10 +345,9 @@ void ej_batch_destroy(ej_batch *batch);
  *     lane per pair, and the warp keeps one ring of x's match masks for all of
  *     them (built cooperatively, once per task) instead of one per lane; pairs
  *     that outlive the rest of their task are left to the persistent verifier.
- *     0 (default): 1 when the strings' mean
- *     length is at least 2048 (long pairs, where refilling pays); else 3 for
- *     alphabets of more than 4 symbols (whose per-lane rings leave the
- *     grid-strided verifier one or two warps per SM) and 2 for the rest.
+ *     0 (default): for alphabets of more than 4 symbols 3 when the strings' mean
+ *     length is below 2048, else 1; for the others 3 when a string is expected to
+ *     share a signature with at least two others by chance, else 1.
  *   chain (batches): how the verifiers of a batch's joins share the GPU: the
  *     persistent ones merged, chained or overlapping, the grid-strided ones
  *     chained unless chain is 1 (the other stages always overlap); see the
@@ -370,7 +369,7 @@ void ej_batch_destroy(ej_batch *batch);
  *     the length filter, have similar lengths); 1: by decreasing number of tables
  *     in which the two strings collided; 2: hash-table order. 0 (default): 4
  *     with the persistent verifier, 3 with the grid-strided one, 5 with the
- *     shared-string one (whose candidates are grouped by a sort, not a hash
+ *     shared-string one (whose candidates come grouped, without a hash
  *     table). In a batch's union launch (chain 0 / 4) the joins' candidates
  *     keep hash order and the union is ordered by the shorter string's length
  *     class, then by the number of joins that list the pair (1: that number

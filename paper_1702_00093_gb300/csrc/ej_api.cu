@@ -707,25 +707,39 @@ constexpr unsigned SMEM_BUCKET_MAX = 256;
 // tables with length windows instead of hashed buckets.
 constexpr unsigned SORTED_BUCKET_MIN = 4096;
 
-// Threads per block of the persistent verifier this join uses, 0 for the
-// grid-strided one. Mode 0 picks the persistent verifier for long strings only
-// (mean length >= 2048): on short, mostly rejected pairs its per-pair refill
-// costs more than it saves (measured 2x slower on the protein-like shape).
-int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
-    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
-    const bool want_pq = ctx->sched.mode == 1 || (ctx->sched.mode == 0 && long_pairs);
-    return (vc.G == 2 && want_pq) ? pq_threads_for(pq_words(p->K), p->alphabet_size) : 0;
+// The verifier of mode 0 (measured as whole joins of 20000 strings unless said).
+// More than four symbols: the shared-string verifier for mean lengths below 2048,
+// else the persistent one. At most four symbols (rings of a few hundred bytes per
+// lane): the shared-string verifier when chance alone fills its tasks, i.e. a string
+// meets at least two others that are unrelated, counted as if the z symbols of a
+// signature were uniform (r m n / 2 alphabet^-z; signatures of short strings
+// coincide more often): 1.8M candidates of 100-base reads (5.3) 5.2 (grid-strided)
+// or 5.5 (persistent) -> 1.15 ms, 1500 bases (5.3) 1.9 -> 1.5, 5000 bases at K = 250
+// (85) 26.4 -> 19.5; the persistent one otherwise: 500 bases (1.3) 1.02 against 1.04
+// ms, 5000 reads of 1000 bases (0.3) 0.37 against 0.75, 5000 bases at K = 150 (0)
+// 0.80 against 1.7.
+bool long_strings(const Plan &pl) { return pl.st.n > 0 && pl.st.total / pl.st.n >= 2048; }
+
+bool dense_signatures(const Plan &pl, const ej_params *p) {
+    double chance = 0.5 * (double)p->r * p->m * (double)pl.st.n;
+    for (uint32_t q = 0; q < p->z && chance >= 2.0; q++) chance /= p->alphabet_size;
+    return chance >= 2.0;
 }
 
-// The shared-string verifier (mode 3; mode 0 for short strings over more than
-// four symbols, whose per-lane match-mask rings would leave the other verifiers
-// a few warps per SM): the band within SX_MAX_WORDS words, the warps' rings within
-// the block's budget.
+// The shared-string verifier: mode 3, or the choice of mode 0; the band within
+// SX_MAX_WORDS words, the warps' rings within the block's budget.
 bool sx_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
     const int W = sx_band(p->K).W;
     if (vc.G != 2 || W > SX_MAX_WORDS || sx_smem_bytes(W, p->alphabet_size) > 220 * 1024) return false;
-    const bool long_pairs = pl.st.n > 0 && pl.st.total / pl.st.n >= 2048;
-    return ctx->sched.mode == 3 || (ctx->sched.mode == 0 && !long_pairs && p->alphabet_size > 4);
+    if (ctx->sched.mode != 0) return ctx->sched.mode == 3;
+    return p->alphabet_size > 4 ? !long_strings(pl) : dense_signatures(pl, p);
+}
+
+// Threads per block of the persistent verifier this join uses, 0 for none.
+int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
+    const bool want_pq = ctx->sched.mode == 1 ||
+                         (ctx->sched.mode == 0 && (long_strings(pl) || p->alphabet_size <= 4) && !sx_choice(ctx, pl, p, vc));
+    return (vc.G == 2 && want_pq) ? pq_threads_for(pq_words(p->K), p->alphabet_size) : 0;
 }
 
 int back_buckets(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *keys, BackState *bs,

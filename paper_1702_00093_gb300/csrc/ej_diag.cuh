@@ -202,6 +202,41 @@ __device__ __forceinline__ int32_t diag_min(const uint32_t (&P)[W], const uint32
     return (int32_t)bound >> 16;
 }
 
+// The same minimum as the return value, and *alive: whether some row may lie on an
+// alignment of cost <= K, judged per half word: T + its minimum + the distance of
+// the half's rows (16 h + 1 .. 16 h + 16 below the top cell, which counts to half 0)
+// to the diagonal on which the alignment ends, rt rows below the top cell, is <= K.
+// On every alignment of cost <= K there is such a row, and random strings run out
+// of them about 7% of the columns before the plain minimum exceeds K.
+template <int W>
+__device__ __forceinline__ int32_t diag_alive(const uint32_t (&P)[W], const uint32_t (&M)[W], const uint32_t *tab,
+                                              int32_t T, int32_t rt, int32_t K, bool *alive) {
+    uint32_t run2 = 0;
+    int32_t low = 0, best = 0x7FFFFFFF;   // smallest minimum, smallest minimum + distance
+#pragma unroll
+    for (int v = 0; v < W; v++) {
+        const uint32_t even = (P[v] & 0x0F0F0F0Fu) | ((M[v] & 0x0F0F0F0Fu) << 4);
+        const uint32_t odd = ((P[v] >> 4) & 0x0F0F0F0Fu) | (M[v] & 0xF0F0F0F0u);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            uint32_t bound = v + h == 0 ? 0x00007FFFu : 0x7FFF7FFFu;
+#pragma unroll
+            for (int k = 4 * h; k < 4 * h + 4; k++) {
+                const uint32_t idx = __byte_perm((k & 1) ? odd : even, 0u, 0x4440 | (k >> 1));
+                const uint32_t x = __viaddmin_s16x2(run2, tab[idx], bound);
+                run2 = __byte_perm(x, 0u, 0x1010);
+                bound = (x & 0xFFFF0000u) | 0x7FFFu;
+            }
+            const int32_t mn = (int32_t)bound >> 16;
+            low = min(low, mn);
+            const int first = 32 * v + 16 * h + (v + h == 0 ? 0 : 1), last = 32 * v + 16 * h + 16;
+            best = min(best, mn + max(max(first - rt, rt - last), 0));
+        }
+    }
+    *alive = T + best <= K;
+    return low;
+}
+
 // Sum of the differences of the first `cnt` rows of a dumped window (entries v
 // and W + v, `stride` apart: words v of P and M).
 template <int W>

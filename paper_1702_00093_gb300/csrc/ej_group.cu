@@ -1,8 +1,9 @@
 // Candidates grouped for the shared-string verifier (Alg. 3's filtering and
 // deduplication): for every string x, the strings y that precede it in (length,
 // id) order, share a signature with it in some table and differ in length by at
-// most K, each once, in warp tasks of up to 32 pairs that share x and the class of
-// the length difference.
+// most K, each once, in warp tasks of up to 32 pairs that share x and two adjacent
+// classes of the length difference (partners come in increasing difference; a task
+// that is not full takes pairs of the next class, so that few leave part empty).
 //
 // Every table's records are sorted by (signature, length, id), so the partners of
 // x in a table are the records of one window just before x's own. A warp takes
@@ -31,6 +32,7 @@ namespace {
 
 constexpr int GE_WARPS = 8;    // warps per block of the emitting kernel
 constexpr int GE_BLOCKS = 8;   // blocks per SM
+constexpr int GE_KEEP = 160;   // tables whose windows are kept from class to class
 
 __device__ __forceinline__ uint32_t fingerprint(uint64_t k) {
     k ^= k >> 31;
@@ -111,6 +113,17 @@ __device__ __forceinline__ uint32_t window_first(const uint64_t *__restrict__ rk
     return good;
 }
 
+// The first record in [lo, end), ascending by length, of at least `lim` as length.
+__device__ __forceinline__ uint32_t lower_len(const uint64_t *__restrict__ rec, uint32_t lo, uint32_t end, int64_t lim) {
+    const uint64_t vlim = lim > 0 ? (uint64_t)lim << 32 : 0ull;
+    while (lo < end) {
+        const uint32_t mid = (lo + end) >> 1;
+        if (rec[mid] >= vlim) end = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
 // x and y share a signature in some table before t: rows fx, fy of fingerprints,
 // equal ones confirmed on the signatures.
 __device__ __forceinline__ bool met_before(const uint4 *__restrict__ fx, const uint4 *__restrict__ fy, int32_t t,
@@ -141,6 +154,9 @@ group_emit_kernel(const uint64_t *__restrict__ rk, const uint64_t *__restrict__ 
     __shared__ uint64_t s_stage[GE_WARPS][64];
     const int lane = threadIdx.x & 31;
     uint64_t *stage = s_stage[threadIdx.x >> 5];
+    // the windows of the first GE_KEEP tables from class to class (own lane's entries)
+    __shared__ uint32_t s_keep[GE_WARPS][2][GE_KEEP];
+    uint32_t *keep_lo = s_keep[threadIdx.x >> 5][0], *keep_end = s_keep[threadIdx.x >> 5][1];
     const int64_t nw = (int64_t)gridDim.x * GE_WARPS;
     unsigned long long raw = 0, kept = 0;
     int64_t tnext = 0, tend = 0;   // the warp's task numbers left of its last reservation
@@ -163,23 +179,42 @@ group_emit_kernel(const uint64_t *__restrict__ rk, const uint64_t *__restrict__ 
     for (int64_t x = (int64_t)blockIdx.x * GE_WARPS + (threadIdx.x >> 5); x < n; x += nw) {   // warp-uniform
         const int64_t lx = lens[x];
         const uint4 *fx = fp + x * FW;
+        int staged = 0;
+        int32_t oldest = 0;   // the class of the first staged pair
         for (int32_t c = 0; c < nclass; c++) {
             // partners of lengths lx - dhi .. lx - dlo
             const int64_t dlo = (int64_t)c * width, dhi = min((int64_t)K, dlo + width - 1);
             if (dlo > lx) break;
-            int staged = 0;
+            if (staged && c > oldest + 1) {   // two classes at most
+                flush(staged);
+                staged = 0;
+            }
             for (int32_t t0 = 0; t0 < T; t0 += 32) {
                 uint32_t first = 0, cnt = 0;
-                if (t0 + lane < T) {
-                    const int64_t tb = (int64_t)(t0 + lane) * n;
-                    const uint32_t p = pos[tb + x];
-                    const uint64_t key = rk[tb + p];
-                    if (p > 0 && rk[tb + p - 1] == key) {
-                        const uint32_t end = c == 0 ? p : window_first(rk + tb, rec + tb, p, key, lx - dlo + 1);
-                        first = window_first(rk + tb, rec + tb, p, key, lx - dhi);
-                        cnt = end - first;
+                const int32_t t = t0 + lane;
+                if (t < T) {
+                    const int64_t tb = (int64_t)t * n;
+                    uint32_t lo = 0, end = 0;   // x's window in the table, without the classes done
+                    if (c == 0 || t >= GE_KEEP) {
+                        const uint32_t p = pos[tb + x];
+                        const uint64_t key = rk[tb + p];
+                        lo = end = p;
+                        if (p > 0 && rk[tb + p - 1] == key) {
+                            lo = window_first(rk + tb, rec + tb, p, key, lx - K);
+                            if (c > 0) end = lower_len(rec + tb, lo, p, lx - dlo + 1);
+                        }
+                    } else {
+                        lo = keep_lo[t];
+                        end = keep_end[t];
+                    }
+                    first = c + 1 < nclass && lo < end ? lower_len(rec + tb, lo, end, lx - dhi) : lo;
+                    cnt = end - first;
+                    if (t < GE_KEEP && nclass > 1) {
+                        keep_lo[t] = lo;
+                        keep_end[t] = first;
                     }
                 }
+                if (!__any_sync(FULL, cnt > 0)) continue;
                 uint32_t incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -202,9 +237,9 @@ group_emit_kernel(const uint64_t *__restrict__ rk, const uint64_t *__restrict__ 
                     bool keep = false;
                     uint32_t y = 0;
                     if (item < total) {
-                        const int32_t t = t0 + l;
-                        y = (uint32_t)rec[(int64_t)t * n + f + (item - ex)];
-                        keep = !met_before(fx, fp + (int64_t)y * FW, t, keys, n, (uint32_t)x, y);
+                        const int32_t ti = t0 + l;
+                        y = (uint32_t)rec[(int64_t)ti * n + f + (item - ex)];
+                        keep = !met_before(fx, fp + (int64_t)y * FW, ti, keys, n, (uint32_t)x, y);
                     }
                     const unsigned mask = __ballot_sync(FULL, keep);
                     if (keep) {
@@ -213,6 +248,7 @@ group_emit_kernel(const uint64_t *__restrict__ rk, const uint64_t *__restrict__ 
                             xi < y ? ((uint64_t)xi << 32) | y : ((uint64_t)y << 32) | xi;
                     }
                     __syncwarp();
+                    if (staged == 0) oldest = c;
                     staged += __popc(mask);
                     if (staged >= 32) {
                         flush(32);
@@ -221,11 +257,12 @@ group_emit_kernel(const uint64_t *__restrict__ rk, const uint64_t *__restrict__ 
                         __syncwarp();
                         if (lane < staged) stage[lane] = rest;
                         __syncwarp();
+                        oldest = c;   // what is left came with the last 32 items
                     }
                 }
             }
-            if (staged) flush(staged);
         }
+        if (staged) flush(staged);
     }
     // reserved and not used
     if (tnext + lane < tend && tnext + lane < tcap) tasks[tnext + lane] = 0u;

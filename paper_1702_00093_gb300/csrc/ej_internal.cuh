@@ -338,7 +338,7 @@ cudaError_t launch_dedup_by_first(const uint64_t *raw, uint64_t cap, uint64_t *t
                                   const int32_t *longer_lens = nullptr);
 // Candidates for the shared-string verifier (ej_group.cu). Task i is tasks[i] <= 32
 // pairs at pairs[32 i ..], all with the same longer string (the later one of two
-// equally long) and length-difference class; counters: [0] raw pairs, [1] largest
+// equally long) and a length difference in one of two adjacent classes; counters: [0] raw pairs, [1] largest
 // bucket, [2] candidates, [7] task numbers in use (beyond tcap nothing is
 // written). group_task_cap: the tasks that cap pairs may need. rk / rid: the
 // tables' records sorted by (signature, length, id); rec, pos: n T entries; fp:
@@ -353,11 +353,11 @@ cudaError_t launch_group_emit(const uint64_t *rk, const uint64_t *rec, const uin
                               uint32_t nclass, int64_t tcap, uint64_t *pairs, uint32_t *tasks,
                               unsigned long long *counters, cudaStream_t s);
 // Shared-string verifier (ej_verify_sx.cu).
-// sx_band(K): the verifier's window of W 32-bit words and the class width and
-// count that keep a task's band within it: a task's length differences lie in
-// one class of width D, so its band (the diagonals a cost-K alignment of any of
-// its pairs can use) spans at most K + (D - 1)/2 + 1 diagonals; D uses the rows
-// that ceil((K + 1) / 32) words leave (at least 7, else one more word).
+// sx_band(K): the verifier's window of W 32-bit words and the classes of the length
+// difference d (d / width, nclass of them). A task's pairs lie in two adjacent
+// classes, so the diagonals a cost-K alignment of any of them can use span at most
+// K + 1 + (2 width - 1) / 2, which the window holds: the width is one more than the
+// diagonals that W words leave beyond K + 1.
 struct SxBand {
     int W;
     uint32_t width, nclass;

@@ -3,12 +3,12 @@
 // shared by a warp.
 //
 // The candidates arrive grouped by x, the longer string of each pair, and by
-// the class of the length difference d = |x| - |y| (sx_band), in warp tasks of
-// up to 32 pairs that all share x and the class, one lane per pair. A path of
+// their length difference d = |x| - |y| (sx_band), in warp tasks of up to 32 pairs
+// that all share x and two adjacent classes of d, one lane per pair. A path of
 // cost <= K of a pair stays on the diagonals i - j in
 // [-floor((K - d)/2), floor((K + d)/2)] (the persistent verifier's band); the
 // task's band is the union of its pairs' bands, at most K + 1 + (D - 1)/2
-// diagonals for a class of width D, held in a diagonal window of W 32-bit words
+// diagonals for differences of a range of D, held in a diagonal window of W 32-bit words
 // (ej_diag.cuh). All pairs of a task start together, so at every column their
 // windows cover the same rows of x: the warp keeps one ring of W + 1 match words
 // per symbol in shared memory. A word is built by the whole warp, every 32
@@ -21,21 +21,23 @@
 // per pair halves the tasks, and with them the rings, the loads and the window
 // minima per pair.
 //
-// Early exit. The window's minimum (ej_diag.cuh) is a lower bound of the
-// distance. It is taken first after 11 K / 8 columns, then when the growth so far
-// says that the slowest of the pairs about to be rejected will be (a multiple of
-// 8 columns). Pairs that are not (similar strings run to the end) would keep the
+// Early exit. A pair is rejected when no row of its window can lie on an alignment
+// of cost <= K (diag_alive). That is looked at first after 9 K / 8 columns, then
+// when the growth so far says that the slowest of the pairs about to be rejected
+// will be (a multiple of 8 columns). Pairs that are not (similar strings run to the end) would keep the
 // warp with most lanes idle: once at most 8 lanes are left and all of them are
 // such, they are appended to a list that the persistent verifier takes from the
 // start (vo.defer; without one the task runs to its end).
 //
 // What bounds it: 32-bit integer instructions, 10 W + about 8 per column and
 // lane, and 5 per window row and quarter for a minimum.
-// 20000 tasks a millisecond and more keep the integer pipe 79% busy (0.59
-// instructions issued a cycle). 622M candidates of 200000 protein-like strings
-// (K = 40, W = 2): 274 -> 77 ms against two lanes per pair on 64-bit block-aligned
-// words with a test every 32 columns; 30M of 120000 text-like strings (K = 200,
-// W = 7): 97.3 -> 41.7 ms and 3.4 ms for the pairs handed over.
+// The integer pipe is 79% busy (0.59 instructions issued a cycle, K = 40). 622M
+// candidates of 200000 protein-like strings (K = 40, W = 2): 274 -> 73 ms against two
+// lanes per pair on 64-bit block-aligned words with a minimum every 32 columns
+// (77 ms with the plain minimum, first after 11 K / 8 columns); 30M of 120000
+// text-like strings (K = 200, W = 7): 97.3 -> 39.1 ms and 3.3 ms for the pairs handed
+// over. Narrowing the window as its outer rows drop out was slower (58.6 ms on text):
+// the rows that some of 32 pairs still needs leave only in the last third.
 #include "ej_diag.cuh"
 
 namespace ej {
@@ -148,7 +150,7 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         else if (valid && n == 0) { running = false; pass = m <= K; }
         int32_t cols_run = 0;
         // the task's band: the diagonals a cost-K alignment of any of its
-        // undecided pairs can use (their length differences lie in one class)
+        // undecided pairs can use (their length differences lie in two classes)
         const unsigned nlo = __reduce_min_sync(FULL, running ? (unsigned)n : 0xFFFFFFFFu);
         const unsigned nhi = __reduce_max_sync(FULL, running ? (unsigned)n : 0u);
         if (nhi > 0) {   // some pair is running
@@ -192,7 +194,7 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             uint32_t sym_next = row_sym<B>(xc, mx, (int64_t)32 * (W + 1) - klo + lane);
             int base = 0;
             int32_t j = 0;                                             // columns done
-            int32_t next_check = (11 * (K >> 3) + 15) & ~7;             // a multiple of 8, above K
+            int32_t next_check = (9 * (K >> 3) + 15) & ~7;              // a multiple of 8, above K
             if (next_check <= K) next_check = (K + 8) & ~7;
             int32_t jend = (int32_t)nlo;                               // the first end of a running pair
             while (true) {
@@ -270,15 +272,17 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
                     if (j < next_check) continue;
                 }
                 // the windows' minima; lanes predicted to be rejected within half as
-                // many columns again keep the task going
-                const int32_t lb = T + diag_min<W>(P, M, s_tab);
-                if (running && lb > K) {
+                // many columns again (a quarter before their minimum would exceed K)
+                // keep the task going
+                bool alive;
+                const int32_t lb = T + diag_alive<W>(P, M, s_tab, T, m - n + klo, K, &alive);
+                if (running && !alive) {
                     running = false;
                     cols_run = j;
                 }
                 const unsigned left = __ballot_sync(FULL, running);
                 if (left == 0u) break;
-                const float rem = (float)(K + 1 - lb) * (float)j / (float)(lb > 1 ? lb : 1);
+                const float rem = 0.75f * (float)(K + 1 - lb) * (float)j / (float)(lb > 1 ? lb : 1);
                 const bool soon = running && rem <= 0.5f * (float)j;
                 const unsigned far = __reduce_max_sync(FULL, soon ? (unsigned)rem + 1u : 0u);
                 if (far > 0u) {
@@ -358,15 +362,16 @@ cudaError_t launch_sx_t(const uint4 *packed, const uint64_t *pofs, const int32_t
 }  // namespace
 
 SxBand sx_band(int32_t K) {
-    const int words = (K + 32) / 32;   // ceil((K + 1) / 32)
-    int W = words, slack = 32 * words - (K + 1);
-    if (2 * slack + 1 < 7) {   // classes narrower than 7 would split the strings' pairs too finely
+    int W = (K + 32) / 32;             // ceil((K + 1) / 32)
+    int slack = 32 * W - (K + 1);      // diagonals the window has beyond a single pair's band
+    if (K > 2 * slack + 1 && (slack + 1 < 4 || K / (slack + 1) + 1 > 16)) {
+        // length differences narrower than 8 split a string's pairs too finely, and
+        // more than 16 classes cost their searches: one word more
         W += 1;
         slack += 32;
     }
-    uint32_t D = 2u * (uint32_t)slack + 1u;
-    if (D > (uint32_t)K + 1u) D = (uint32_t)K + 1u;
-    return SxBand{W, D, ((uint32_t)K + 1u + D - 1u) / D};
+    if (K <= 2 * slack + 1) return SxBand{W, (uint32_t)K + 1u, 1u};   // every difference fits one task
+    return SxBand{W, (uint32_t)slack + 1u, (uint32_t)K / ((uint32_t)slack + 1u) + 1u};
 }
 
 size_t sx_smem_bytes(int W, uint32_t alpha) { return (size_t)alpha * sx_row(W) * sizeof(uint32_t) * SX_WARPS; }
