@@ -211,7 +211,9 @@ int ej_measure_int_peak(int device, int32_t mix, int32_t iters, double *ops_per_
  * the index strings s that share a signature with q in some table, pass
  * ||q| - |s|| <= K[q] and have ED(q, s) <= K[q] (the join's candidate rule and
  * test, from the query's side). Output: (q << 32 | s) ascending, q = query
- * position, s = index position. Synchronous (one search batch; stream unused).
+ * position, s = index position. Synchronous (one search batch; stream unused). The
+ * index keeps the scratch of up to two searches (1 GiB each at most) between calls;
+ * calls that run at the same time never share one.
  * Errors: EJ_ERR_INVALID_ARG (a query byte outside the alphabet, bad offsets,
  * K < 0, device query buffers), EJ_ERR_CAPACITY (*n_out = needed).
  */

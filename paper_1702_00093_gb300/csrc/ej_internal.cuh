@@ -325,7 +325,8 @@ cudaError_t launch_index_runs(const uint64_t *rk, const uint32_t *rid, const int
 cudaError_t launch_index_probe(const uint64_t *qkeys, int64_t Q, int64_t T, const int32_t *qlens, const int32_t *qK,
                                const uint64_t *slot_keys, const uint2 *runs, uint64_t H, const uint64_t *rec,
                                int64_t n, uint64_t *raw, uint64_t cap, unsigned long long *counters, cudaStream_t s);
-cudaError_t launch_dedup_classes(const uint64_t *raw, uint64_t cap, uint64_t *table, uint32_t *hcount, uint64_t hsize,
+// uniq: cap entries; with one class (nc = 1) the pairs go to cand at once.
+cudaError_t launch_dedup_classes(const uint64_t *raw, uint64_t cap, uint64_t *table, uint64_t *uniq, uint64_t hsize,
                                  const uint8_t *cls, int nc, unsigned long long *bins, uint64_t *cand,
                                  unsigned long long *counters, cudaStream_t s);
 // Dedup ordered by the pair's first string (counting sort over n bins): bins

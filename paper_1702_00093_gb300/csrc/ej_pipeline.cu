@@ -1013,19 +1013,55 @@ cudaError_t launch_index_probe(const uint64_t *qkeys, int64_t Q, int64_t T, cons
 
 // Dedup of query x index pairs, grouped by the verifier class of the query:
 // bins[c] = pairs of class c, bins[nc + c] = their start in cand (classes in
-// order), counters[2] = all pairs. bins (3*nc) and hcount start at zero.
-__global__ void class_hist_kernel(const uint64_t *__restrict__ table, uint64_t hsize, const uint8_t *__restrict__ cls,
-                                  unsigned long long *__restrict__ bins, unsigned long long *__restrict__ counters) {
-    unsigned int mine = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)hsize; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t key = table[i];
-        if (key != ~0ull) {
-            atomicAdd(&bins[cls[key >> 32]], 1ull);
-            mine++;
+// order), counters[2] = all pairs. bins (3*nc) start at zero, table at ~0. The first
+// copy of every pair is appended to uniq as it enters the table (so nothing scans
+// the table afterwards) and counted to its class in shared memory; the scatter
+// takes one place per class and warp (one atomic per pair on a handful of class
+// cursors took 0.64 ms for 200000 pairs, and as much again to count them).
+__global__ void __launch_bounds__(256)
+dedup_classes_kernel(const uint64_t *__restrict__ raw, uint64_t cap, uint64_t *__restrict__ table, uint64_t hsize,
+                     const uint8_t *__restrict__ cls, int nc, uint64_t *__restrict__ uniq,
+                     unsigned long long *__restrict__ bins, unsigned long long *__restrict__ counters) {
+    __shared__ unsigned int sb[256];   // classes are 8-bit
+    for (int t = threadIdx.x; t < 256; t += blockDim.x) sb[t] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const unsigned long long nraw_all = counters[0];
+    const int64_t nraw = (int64_t)(nraw_all < cap ? nraw_all : cap);
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t start = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t iters = (nraw + step - 1) / step;   // the same on every lane
+    for (int64_t it = 0; it < iters; it++) {
+        const int64_t i = start + it * step;
+        bool is_new = false;
+        uint64_t key = 0;
+        if (i < nraw) {
+            key = raw[i];
+            uint64_t h = pair_hash(key) & (hsize - 1);
+            for (uint64_t probe = 0; probe < hsize; probe++) {
+                const unsigned long long old = atomicCAS((unsigned long long *)&table[h], ~0ull, key);
+                if (old == ~0ull) {
+                    is_new = true;
+                    break;
+                }
+                if (old == key) break;
+                h = (h + 1) & (hsize - 1);
+            }
+        }
+        const unsigned mask = __ballot_sync(FULL, is_new);
+        if (mask) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(&counters[2], (unsigned long long)__popc(mask));
+            base = __shfl_sync(FULL, base, 0);
+            if (is_new) {
+                uniq[base + __popc(mask & ((1u << lane) - 1u))] = key;
+                atomicAdd(&sb[cls[key >> 32]], 1u);
+            }
         }
     }
-    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(FULL, mine, o);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&counters[2], (unsigned long long)mine);
+    __syncthreads();
+    for (int t = threadIdx.x; t < nc; t += blockDim.x)
+        if (sb[t]) atomicAdd(&bins[t], (unsigned long long)sb[t]);
 }
 
 __global__ void class_scan_kernel(unsigned long long *__restrict__ bins, int nc) {
@@ -1039,26 +1075,41 @@ __global__ void class_scan_kernel(unsigned long long *__restrict__ bins, int nc)
     }
 }
 
-__global__ void class_scatter_kernel(const uint64_t *__restrict__ table, uint64_t hsize,
-                                     const uint8_t *__restrict__ cls, unsigned long long *__restrict__ cursor,
-                                     uint64_t *__restrict__ cand) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)hsize; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t key = table[i];
-        if (key != ~0ull) cand[atomicAdd(&cursor[cls[key >> 32]], 1ull)] = key;
+__global__ void __launch_bounds__(256)
+class_scatter_kernel(const uint64_t *__restrict__ uniq, uint64_t cap, const uint8_t *__restrict__ cls,
+                     unsigned long long *__restrict__ cursor, uint64_t *__restrict__ cand,
+                     const unsigned long long *__restrict__ counters) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nu = (int64_t)(counters[2] < cap ? counters[2] : cap);
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t start = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t iters = (nu + step - 1) / step;   // the same on every lane
+    for (int64_t it = 0; it < iters; it++) {
+        const int64_t i = start + it * step;
+        const uint64_t key = i < nu ? uniq[i] : 0ull;
+        const uint32_t c = i < nu ? cls[key >> 32] : 256u;
+        const unsigned peers = __match_any_sync(FULL, c);
+        const int leader = __ffs(peers) - 1;
+        unsigned long long base = 0;
+        if (lane == leader && c < 256u) base = atomicAdd(&cursor[c], (unsigned long long)__popc(peers));
+        base = __shfl_sync(FULL, base, leader);
+        if (c < 256u) cand[base + __popc(peers & ((1u << lane) - 1u))] = key;
     }
 }
 
-cudaError_t launch_dedup_classes(const uint64_t *raw, uint64_t cap, uint64_t *table, uint32_t *hcount, uint64_t hsize,
+cudaError_t launch_dedup_classes(const uint64_t *raw, uint64_t cap, uint64_t *table, uint64_t *uniq, uint64_t hsize,
                                  const uint8_t *cls, int nc, unsigned long long *bins, uint64_t *cand,
                                  unsigned long long *counters, cudaStream_t s) {
-    int64_t g = ((int64_t)cap + 255) / 256;
-    dedup_count_kernel<<<(unsigned)(g > 8192 ? 8192 : (g ? g : 1)), 256, 0, s>>>(raw, cap, table, hcount, hsize, counters);
-    int64_t gh = ((int64_t)hsize + 255) / 256;
-    const unsigned gs = (unsigned)(gh > 2048 ? 2048 : (gh ? gh : 1));
-    class_hist_kernel<<<gs, 256, 0, s>>>(table, hsize, cls, bins, counters);
-    class_scan_kernel<<<1, 32, 0, s>>>(bins, nc);
-    class_scatter_kernel<<<gs, 256, 0, s>>>(table, hsize, cls, bins + 2 * nc, cand);
-    note_launches(4);
+    if (nc < 1 || nc > 256) return cudaErrorInvalidValue;
+    const int64_t g = ((int64_t)cap + 255) / 256;
+    const unsigned gs = (unsigned)(g > 152 * 8 ? 152 * 8 : (g ? g : 1));
+    dedup_classes_kernel<<<gs, 256, 0, s>>>(raw, cap, table, hsize, cls, nc, nc == 1 ? cand : uniq, bins, counters);
+    note_launches(1);
+    if (nc > 1) {
+        class_scan_kernel<<<1, 32, 0, s>>>(bins, nc);
+        class_scatter_kernel<<<gs, 256, 0, s>>>(uniq, cap, cls, bins + 2 * nc, cand, counters);
+        note_launches(2);
+    }
     return cudaGetLastError();
 }
 

@@ -71,13 +71,57 @@ T *P(const DevBuf &b) {
     return (T *)b.p;
 }
 
-int words_for(int32_t K) { return (2 * K + 1 + 63) / 64; }
+// Window class of a query: the persistent verifier's words, beyond its reach the
+// words of Ukkonen's band (their classes are more than 24).
+int sv_class(int32_t K) {
+    const int w = pq_words(K);
+    return w <= PQ_MAX_WORDS ? w : (2 * K + 1 + 63) / 64 + PQ_MAX_WORDS;
+}
 
 #define SV(expr)                                              \
     do {                                                      \
         cudaError_t e_ = (expr);                              \
         if (e_ != cudaSuccess) return e_;                     \
     } while (0)
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// One search batch in flight
+// ---------------------------------------------------------------------------
+
+namespace {
+
+struct Slot {
+    cudaStream_t s = nullptr;
+    cudaEvent_t done = nullptr;
+    DevBuf in, qlens, ccnt, qpofs, scan, qpacked, qkeys, raw, table, uniq, bins, cand, app, cnt, derr, queue, tickets;
+    void *h_in = nullptr;
+    size_t h_in_bytes = 0;
+    unsigned long long *h_out = nullptr;   // counters[8], error word, then the result prefix
+    size_t h_out_entries = 0;
+    uint64_t cap = 1 << 16;                // raw / candidate / output capacity
+    // the batch
+    int64_t Q = 0;
+    size_t pre = 0;                        // results copied back with its counters
+    size_t device_bytes = 0;
+};
+
+constexpr size_t kOutHead = 16;            // u64 words before the result prefix
+constexpr size_t kPrefix = 1 << 16;        // results copied back with the counters, at most
+constexpr size_t kPoolSlots = 2;
+constexpr size_t kPoolBytes = (size_t)1 << 30;
+
+void slot_free(Slot &sl) {
+    for (DevBuf *b : {&sl.in, &sl.qlens, &sl.ccnt, &sl.qpofs, &sl.scan, &sl.qpacked, &sl.qkeys, &sl.raw, &sl.table,
+                      &sl.uniq, &sl.bins, &sl.cand, &sl.app, &sl.cnt, &sl.derr, &sl.queue, &sl.tickets})
+        dev_free(*b);
+    if (sl.h_in) cudaFreeHost(sl.h_in);
+    if (sl.h_out) cudaFreeHost(sl.h_out);
+    if (sl.done) cudaEventDestroy(sl.done);
+    if (sl.s) cudaStreamDestroy(sl.s);
+    sl = Slot{};
+}
 
 }  // namespace
 
@@ -96,6 +140,10 @@ struct ej_index {
     uint64_t H = 0;
     bool use_table = false;
     DevBuf pos, tsym, spos, stag, next, skeys, runs, rec, err;
+    // search slots between calls of ej_index_search (a search takes one or makes
+    // one: concurrent calls never share), at most kPoolSlots of kPoolBytes each
+    std::mutex pool_mu;
+    std::vector<Slot> pool;
 };
 
 namespace {
@@ -104,47 +152,16 @@ void index_free(ej_index *x) {
     if (!x) return;
     for (DevBuf *b : {&x->pos, &x->tsym, &x->spos, &x->stag, &x->next, &x->skeys, &x->runs, &x->rec, &x->err})
         dev_free(*b);
+    for (Slot &sl : x->pool) slot_free(sl);
     if (x->own) ej_destroy(x->own);
     delete x;
 }
-
-// ---------------------------------------------------------------------------
-// One search batch in flight
-// ---------------------------------------------------------------------------
 
 struct Query {
     const uint8_t *bytes;
     int32_t len;
     int32_t K;
 };
-
-struct Slot {
-    cudaStream_t s = nullptr;
-    cudaEvent_t done = nullptr;
-    DevBuf in, qlens, ccnt, qpofs, scan, qpacked, qkeys, raw, table, hcount, bins, cand, app, cnt, derr, queue, tickets;
-    void *h_in = nullptr;
-    size_t h_in_bytes = 0;
-    unsigned long long *h_out = nullptr;   // counters[8], error word, then the result prefix
-    size_t h_out_entries = 0;
-    uint64_t cap = 1 << 16;                // raw / candidate / output capacity
-    // the batch
-    int64_t Q = 0;
-    size_t device_bytes = 0;
-};
-
-constexpr size_t kOutHead = 16;            // u64 words before the result prefix
-constexpr size_t kPrefix = 1 << 16;        // results copied back with the counters
-
-void slot_free(Slot &sl) {
-    for (DevBuf *b : {&sl.in, &sl.qlens, &sl.ccnt, &sl.qpofs, &sl.scan, &sl.qpacked, &sl.qkeys, &sl.raw, &sl.table,
-                      &sl.hcount, &sl.bins, &sl.cand, &sl.app, &sl.cnt, &sl.derr, &sl.queue, &sl.tickets})
-        dev_free(*b);
-    if (sl.h_in) cudaFreeHost(sl.h_in);
-    if (sl.h_out) cudaFreeHost(sl.h_out);
-    if (sl.done) cudaEventDestroy(sl.done);
-    if (sl.s) cudaStreamDestroy(sl.s);
-    sl = Slot{};
-}
 
 cudaError_t slot_init(Slot &sl) {
     SV(cudaStreamCreateWithFlags(&sl.s, cudaStreamNonBlocking));
@@ -167,9 +184,9 @@ size_t slot_growth(const Slot &sl, const ej_index &x, int64_t Q, int64_t total, 
     const size_t need[] = {
         (size_t)total + (size_t)(Q + 1) * 8 + (size_t)Q * 5 + 64, (size_t)Q * 4, (size_t)(Q + 1) * 4,
         (size_t)(Q + 2) * 8, scan_temp_bytes(Q + 1), (size_t)chunk_bound * 16, (size_t)x.T * Q * 8, cap * 8,
-        hs * 8, hs * 4, 0, cap * 8, cap * 8};
+        hs * 8, cap * 8, 0, cap * 8, cap * 8};
     const DevBuf *have[] = {&sl.in, &sl.qlens, &sl.ccnt, &sl.qpofs, &sl.scan, &sl.qpacked, &sl.qkeys, &sl.raw,
-                            &sl.table, &sl.hcount, &sl.bins, &sl.cand, &sl.app};
+                            &sl.table, &sl.uniq, &sl.bins, &sl.cand, &sl.app};
     size_t g = 0;
     for (size_t i = 0; i < sizeof(need) / sizeof(need[0]); i++)
         if (need[i] > have[i]->bytes) g += need[i];
@@ -200,7 +217,7 @@ cudaError_t slot_reserve(Slot &sl, const ej_index &x, int64_t Q, int64_t total, 
     SV(dev_grow(sl.qkeys, (size_t)x.T * Q * 8, &grown));
     SV(dev_grow(sl.raw, cap * 8, &grown));
     SV(dev_grow(sl.table, hs * 8, &grown));
-    SV(dev_grow(sl.hcount, hs * 4, &grown));
+    SV(dev_grow(sl.uniq, cap * 8, &grown));
     SV(dev_grow(sl.bins, (size_t)3 * nc * 8, &grown));
     SV(dev_grow(sl.cand, cap * 8, &grown));
     SV(dev_grow(sl.app, cap * 8, &grown));
@@ -223,9 +240,9 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
         total += q.len;
         max_q = std::max(max_q, q.len);
     }
-    // window classes: W1 = words(K) + 1 per query, classes in increasing W1
+    // window classes: the persistent verifier's words per query, in increasing order
     std::vector<int> w1s;
-    for (const Query &q : qs) w1s.push_back(words_for(q.K) + 1);
+    for (const Query &q : qs) w1s.push_back(sv_class(q.K));
     std::vector<int> cls_w1 = w1s;
     std::sort(cls_w1.begin(), cls_w1.end());
     cls_w1.erase(std::unique(cls_w1.begin(), cls_w1.end()), cls_w1.end());
@@ -270,7 +287,6 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     SV(cudaMemsetAsync(cnt, 0, 8 * 8, s));
     SV(cudaMemsetAsync(derr, 0, 16, s));
     SV(cudaMemsetAsync(sl.table.p, 0xFF, hs * 8, s));
-    SV(cudaMemsetAsync(sl.hcount.p, 0, hs * 4, s));
     SV(cudaMemsetAsync(bins, 0, (size_t)3 * nc * 8, s));
     SV(cudaMemsetAsync(sl.queue.p, 0, (size_t)nc * 8, s));
     SV(cudaMemsetAsync(sl.tickets.p, 0, (size_t)nc * SM_TICKETS * 4, s));
@@ -288,7 +304,7 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     // buckets -> pairs -> dedup by class
     SV(launch_index_probe(P<uint64_t>(sl.qkeys), Q, x.T, P<int32_t>(sl.qlens), qK, P<uint64_t>(x.skeys),
                           P<uint2>(x.runs), x.H, P<uint64_t>(x.rec), x.set.n, P<uint64_t>(sl.raw), cap, cnt, s));
-    SV(launch_dedup_classes(P<uint64_t>(sl.raw), cap, P<uint64_t>(sl.table), P<uint32_t>(sl.hcount), hs, qcls, nc,
+    SV(launch_dedup_classes(P<uint64_t>(sl.raw), cap, P<uint64_t>(sl.table), P<uint64_t>(sl.uniq), hs, qcls, nc,
                             bins, P<uint64_t>(sl.cand), cnt, s));
     // verify, one launch per window class
     const uint32_t alpha = x.p.alphabet_size;
@@ -324,13 +340,13 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     // counters, error word and the first results back to the host
     SV(cudaMemcpyAsync(sl.h_out, cnt, 8 * 8, cudaMemcpyDeviceToHost, s));
     SV(cudaMemcpyAsync(sl.h_out + 8, derr, 16, cudaMemcpyDeviceToHost, s));
-    const size_t pre = std::min<size_t>(cap, sl.h_out_entries);
-    SV(cudaMemcpyAsync(sl.h_out + kOutHead, sl.app.p, pre * 8, cudaMemcpyDeviceToHost, s));
+    sl.pre = std::min<size_t>(std::min<size_t>(cap, sl.h_out_entries), 1024 + 16 * (size_t)Q);
+    SV(cudaMemcpyAsync(sl.h_out + kOutHead, sl.app.p, sl.pre * 8, cudaMemcpyDeviceToHost, s));
     SV(cudaEventRecord(sl.done, s));
     return cudaSuccess;
 }
 
-enum CollectStatus { COLLECT_OK = 0, COLLECT_RETRY = 1, COLLECT_ERROR = 2 };
+enum CollectStatus { COLLECT_OK = 0, COLLECT_RETRY = 1, COLLECT_ERROR = 2, COLLECT_INVALID = 3 };
 
 // After sl.done: the sorted result pairs (q << 32 | index id) of the batch.
 CollectStatus slot_collect(Slot &sl, std::vector<uint64_t> *pairs, std::string *why) {
@@ -338,8 +354,8 @@ CollectStatus slot_collect(Slot &sl, std::vector<uint64_t> *pairs, std::string *
     const unsigned long long raw = h[0], nout = h[3];
     const uint32_t err = (uint32_t)(h[8] & 0xffffffffull);
     if (err & (DERR_OFFSETS | DERR_SYMBOL)) {
-        *why = "a query failed validation";
-        return COLLECT_ERROR;
+        *why = "a query byte is not in the index's alphabet";
+        return COLLECT_INVALID;
     }
     if (err & DERR_TIMEOUT) {
         *why = "the persistent verifier gave up after its bound of loop passes";
@@ -354,7 +370,7 @@ CollectStatus slot_collect(Slot &sl, std::vector<uint64_t> *pairs, std::string *
         return COLLECT_RETRY;
     }
     pairs->resize(nout);
-    const size_t pre = std::min<size_t>(std::min<size_t>(sl.cap, sl.h_out_entries), nout);
+    const size_t pre = std::min<size_t>(sl.pre, nout);
     if (pre) memcpy(pairs->data(), h + kOutHead, pre * 8);
     if (nout > pre) {
         if (cudaMemcpy(pairs->data() + pre, P<uint64_t>(sl.app) + pre, (nout - pre) * 8, cudaMemcpyDeviceToHost) !=
@@ -484,13 +500,22 @@ int ej_index_search(ej_ctx *ctx, ej_index *x, const ej_strings *queries, const i
         const int64_t a = queries->offsets[i], b = queries->offsets[i + 1];
         if (a < 0 || b < a || b - a >= (1ll << 31) || K[i] < 0)
             return ctx_fail(ctx, EJ_ERR_INVALID_ARG, "invalid query offsets or K");
-        qs[(size_t)i] = Query{queries->bytes + a, (int32_t)(b - a), K[i]};
-        if (!valid_query(*x, qs[(size_t)i].bytes, qs[(size_t)i].len))
-            return ctx_fail(ctx, EJ_ERR_INVALID_ARG, "a query byte is not in the index's alphabet");
+        qs[(size_t)i] = Query{queries->bytes + a, (int32_t)(b - a), K[i]};   // bytes checked as they are packed
     }
     cudaSetDevice(x->device);
     Slot sl;
-    cudaError_t e = slot_init(sl);
+    bool pooled = false;
+    {
+        std::lock_guard<std::mutex> lk(x->pool_mu);
+        if (!x->pool.empty()) {
+            sl = x->pool.back();
+            x->pool.pop_back();
+            pooled = true;
+        }
+    }
+    cudaError_t e = pooled ? cudaSuccess : slot_init(sl);
+    // room for some hundred candidates per query before the first retry
+    sl.cap = std::max<uint64_t>(sl.cap, std::min<uint64_t>(256 * (uint64_t)queries->n, (uint64_t)1 << 22));
     std::vector<uint64_t> pairs;
     std::string why;
     CollectStatus cs = COLLECT_RETRY;
@@ -499,8 +524,17 @@ int ej_index_search(ej_ctx *ctx, ej_index *x, const ej_strings *queries, const i
         if (e == cudaSuccess) e = cudaEventSynchronize(sl.done);
         if (e == cudaSuccess) cs = slot_collect(sl, &pairs, &why);
     }
+    {
+        // kept for the next search with its scratch (never after an error)
+        std::lock_guard<std::mutex> lk(x->pool_mu);
+        if (e == cudaSuccess && sl.device_bytes <= kPoolBytes && x->pool.size() < kPoolSlots) {
+            x->pool.push_back(sl);
+            sl = Slot{};
+        }
+    }
     slot_free(sl);
     if (e != cudaSuccess) return ctx_fail(ctx, EJ_ERR_CUDA, cudaGetErrorString(e));
+    if (cs == COLLECT_INVALID) return ctx_fail(ctx, EJ_ERR_INVALID_ARG, why.c_str());
     if (cs != COLLECT_OK) return ctx_fail(ctx, EJ_ERR_CUDA, cs == COLLECT_RETRY ? "raw pairs kept growing" : why.c_str());
     *n_out = (int64_t)pairs.size();
     if ((int64_t)pairs.size() > capacity) {
@@ -603,7 +637,7 @@ void server_loop(ej_server *srv) {
                 }
                 srv->t_last = now;
             }
-            if (cs == COLLECT_ERROR) srv->last_error = why;
+            if (cs == COLLECT_ERROR || cs == COLLECT_INVALID) srv->last_error = why;
             ss.busy = false;
             ss.batch.clear();
             srv->cv_done.notify_all();
