@@ -30,7 +30,7 @@ enum BufId {
     B_PACKED, B_CHUNK_CNT, B_POFS, B_SCAN_TMP3, B_TSYM, B_SPOS, B_STAG,
     B_HASH, B_APP, B_JCOUNT, B_NEXT, B_HCOUNT, B_BINS, B_TICKETS, B_BKEYS, B_BHEADS, B_BNEXT, B_FBINS, B_FSTARTS,
     B_FSCAN,
-    B_PLUS_SUBLEN, B_PLUS_WHOLE, B_PLUS_SUBOFF, B_PLUS_BYTES, B_PLUS_SCAN, B_PLUS_CAND,
+    B_PLUS_WHOLE, B_PLUS_START, B_PLUS_CAND,
     B_SX_TASKS, B_GREC, B_GPOS, B_GFP,
     B_GROUP_IDX, B_GROUP_OFF, B_GROUP_BYTES, B_GROUP_OUT,
     B_NUM
@@ -253,8 +253,6 @@ int make_plan(ej_ctx *ctx, const ej_strings *S, const ej_params *p, bool need_ls
     CKS(ensure_t(ctx, B_LENS, (size_t)(n > 0 ? n : 1), &pl->lens));
     unsigned long long *dmax = (unsigned long long *)(derr + 2);
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[6], s));
-    CK(launch_validate(pl->st.bytes, pl->st.offsets, n, total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl->lens,
-                       derr, dmax, s));
     // pack into B-bit codes: chunk counts -> offsets -> pack (flags bad symbols)
     pl->B = packed_bits_for(p->alphabet_size);
     uint32_t *ccnt = nullptr;
@@ -266,7 +264,7 @@ int make_plan(ej_ctx *ctx, const ej_strings *S, const ej_params *p, bool need_ls
     CKS(ensure(ctx, B_SCAN_TMP3, scan_temp_bytes(n + 1), &stmp));
     const int64_t chunk_bound = (total * pl->B + 127) / 128 + n + 1;
     CKS(ensure_t(ctx, B_PACKED, (size_t)chunk_bound, &packed));
-    CK(launch_chunk_counts(pl->lens, n, pl->B, ccnt, s));
+    CK(launch_validate(pl->st.bytes, pl->st.offsets, n, total, pl->B, pl->lens, ccnt, derr, dmax, s));
     CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, stmp, s));
     CK(launch_pack(pl->st.bytes, pl->st.offsets, pl->lens, n, total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl->B,
                    pofs, packed, derr, s));
@@ -313,10 +311,8 @@ int plan_device(ej_ctx *ctx, const Plan &pl, cudaStream_t s) {
     uint32_t *derr = (uint32_t *)ctx->bufs[B_DERR].p;
     CK(cudaMemsetAsync(derr, 0, 4 * sizeof(uint32_t), s));
     unsigned long long *dmax = (unsigned long long *)(derr + 2);
-    CK(launch_validate(pl.st.bytes, pl.st.offsets, n, pl.st.total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl.lens,
-                       derr, dmax, s));
     uint32_t *ccnt = (uint32_t *)ctx->bufs[B_CHUNK_CNT].p;
-    CK(launch_chunk_counts(pl.lens, n, pl.B, ccnt, s));
+    CK(launch_validate(pl.st.bytes, pl.st.offsets, n, pl.st.total, pl.B, pl.lens, ccnt, derr, dmax, s));
     CK(exclusive_scan_u32(ccnt, (uint64_t *)pl.pofs, n + 1, nullptr, ctx->bufs[B_SCAN_TMP3].p, s));
     CK(launch_pack(pl.st.bytes, pl.st.offsets, pl.lens, n, pl.st.total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl.B,
                    pl.pofs, (uint4 *)pl.packed, derr, s));
@@ -2034,36 +2030,42 @@ int ej_join_plus(ej_ctx *ctx, const ej_strings *S, const ej_params *p, int32_t d
     const int64_t nq = n * (int64_t)nsub, TT = (int64_t)p->r * p->m;
     if (nq >= (1ll << 31) || nq * TT >= 0xFFFFFFFFll)
         return fail(ctx, EJ_ERR_UNSUPPORTED, "strings x substrings x tables beyond the 32-bit record ids");
-    // the suffix set
-    uint32_t *sub_len = nullptr;
-    int32_t *whole = nullptr;
-    uint64_t *sub_off = nullptr;
-    void *scan = nullptr;
-    CKS(ensure_t(ctx, B_PLUS_SUBLEN, (size_t)nq + 1, &sub_len));
-    CKS(ensure_t(ctx, B_PLUS_WHOLE, (size_t)nq, &whole));
-    CKS(ensure_t(ctx, B_PLUS_SUBOFF, (size_t)nq + 1, &sub_off));
-    CKS(ensure(ctx, B_PLUS_SCAN, scan_temp_bytes(nq + 1), &scan));
-    CK(cudaMemsetAsync(sub_len + nq, 0, sizeof(uint32_t), s));
-    CK(launch_suffix_lengths(pl.lens, n, nsub, delta, sub_len, whole, s));
-    CK(exclusive_scan_u32(sub_len, sub_off, nq + 1, nullptr, scan, s));
-    CK(cudaMemcpyAsync(ctx->h_cnt, sub_off + nq, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    const int64_t sub_total = ctx->h_cnt[0];
-    uint8_t *sub_bytes = nullptr;
-    CKS(ensure_t(ctx, B_PLUS_BYTES, (size_t)(sub_total > 0 ? sub_total : 1), &sub_bytes));
-    CK(launch_suffix_copy(pl.st.bytes, pl.st.offsets, n, nsub, delta, sub_off, sub_bytes, s));
+    // the suffix records, packed from their places in the strings
     if (!ctx->plus_sub && ej_create(&ctx->plus_sub, ctx->device) != EJ_OK)
         return fail(ctx, EJ_ERR_OOM, "suffix-set context");
     ej_ctx *sub = ctx->plus_sub;
     sub->sched = ctx->sched;
-    ej_strings sset{sub_bytes, (const int64_t *)sub_off, nq};
-    ej_params sp = *p;
-    sp.out_len = pl.out_len;   // the whole strings' embedding length and sampling range
-    sp.L = pl.L;
-    Plan spl;
     auto sub_fail = [&](int st) { return fail(ctx, st, "suffix set: %s", sub->err.c_str()); };
-    int st = make_plan(sub, &sset, &sp, true, &spl, s);
+    int32_t *whole = nullptr;
+    int64_t *start = nullptr;
+    CKS(ensure_t(ctx, B_PLUS_WHOLE, (size_t)nq, &whole));
+    CKS(ensure_t(ctx, B_PLUS_START, (size_t)nq, &start));
+    Plan spl = pl;             // the whole strings' embedding length and sampling range
+    spl.st.n = nq;
+    spl.nb32 = (nq + 31) / 32;
+    ej_params sp = *p;
+    sp.out_len = pl.out_len;
+    sp.L = pl.L;
+    int st = upload_alphabet(sub, &sp, s);
+    uint32_t *counts = nullptr;
+    uint64_t *spofs = nullptr;
+    uint4 *spacked = nullptr;
+    void *stmp0 = nullptr;
+    if (st == EJ_OK) st = ensure_t(sub, B_DERR, 8, (uint32_t **)&stmp0);
+    if (st == EJ_OK) st = ensure_t(sub, B_LENS, (size_t)nq, &spl.lens);
+    if (st == EJ_OK) st = ensure_t(sub, B_CHUNK_CNT, (size_t)nq + 1, &counts);
+    if (st == EJ_OK) st = ensure_t(sub, B_POFS, (size_t)nq + 2, &spofs);
+    if (st == EJ_OK) st = ensure(sub, B_SCAN_TMP3, scan_temp_bytes(nq + 1), &stmp0);
+    // no suffix has more chunks than its string
+    const int64_t chunk_bound = nsub * ((pl.st.total * pl.B + 127) / 128 + n) + 1;
+    if (st == EJ_OK) st = ensure_t(sub, B_PACKED, (size_t)chunk_bound, &spacked);
     if (st != EJ_OK) return sub_fail(st);
+    CK(launch_suffix_records(pl.lens, pl.st.offsets, n, nsub, delta, pl.B, spl.lens, counts, start, whole, s));
+    CK(exclusive_scan_u32(counts, spofs, nq + 1, nullptr, stmp0, s));
+    CK(launch_pack(pl.st.bytes, start, spl.lens, nq, pl.st.total, (const uint8_t *)sub->bufs[B_CODEMAP].p, pl.B, spofs,
+                   spacked, (uint32_t *)sub->bufs[B_DERR].p, s));
+    spl.packed = spacked;
+    spl.pofs = spofs;
     uint64_t *keys = nullptr;
     if ((st = ensure_t(sub, B_KEYS, (size_t)(TT * nq), &keys)) != EJ_OK) return sub_fail(st);
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[1], s));

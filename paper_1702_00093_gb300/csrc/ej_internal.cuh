@@ -104,11 +104,11 @@ enum : uint32_t {
 // Kernel launchers (each returns cudaGetLastError() of its launch)
 // ---------------------------------------------------------------------------
 
-// Validation + lengths: lens[i] = offsets[i+1]-offsets[i]; err |= DERR_*;
-// stats[0] = max length (int64 via unsigned max), stats[1] = total bytes.
+// Validation + lengths: lens[i] = offsets[i+1]-offsets[i], counts[i] = its chunks
+// of B-bit codes (counts[n] = 0); err |= DERR_*; *max_len = max length.
 cudaError_t launch_validate(const uint8_t *bytes, const int64_t *offsets, int64_t n, int64_t total_cap,
-                            const uint8_t *code_map, int32_t *lens, uint32_t *err,
-                            unsigned long long *max_len, cudaStream_t s);
+                            int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
+                            cudaStream_t s);
 
 // Random-bit table [r][out_len][words]: bit c of row (l, j) = pi_j^l(alphabet[c]).
 cudaError_t launch_bit_table(uint64_t seed, uint32_t r, uint32_t out_len, const uint8_t *alphabet_dev,
@@ -119,9 +119,8 @@ cudaError_t launch_bit_table(uint64_t seed, uint32_t r, uint32_t out_len, const 
 cudaError_t launch_positions(uint64_t seed, uint32_t r, uint32_t m, uint32_t z, uint32_t L,
                              const uint32_t *pos_inject, uint32_t *pos, cudaStream_t s);
 
-// Chunk counts per string (u32) from lengths.
-cudaError_t launch_chunk_counts(const int32_t *lens, int64_t n, int B, uint32_t *counts, cudaStream_t s);
-// Pack bytes -> codes; bytes outside the alphabet set DERR_SYMBOL (code 0 is stored).
+// Pack bytes -> codes; bytes outside the alphabet set DERR_SYMBOL (some code of the
+// alphabet is stored).
 // total: bytes in the array (every validated string lies inside [0, total)).
 cudaError_t launch_pack(const uint8_t *bytes, const int64_t *offsets, const int32_t *lens, int64_t n, int64_t total,
                         const uint8_t *code_map, int B, const uint64_t *pofs, uint4 *packed,
@@ -240,12 +239,10 @@ cudaError_t launch_compact_u64(const uint64_t *in, const uint8_t *flags, const u
 cudaError_t launch_emit_append(const uint64_t *rec_keys, const uint32_t *rec_ids, const int32_t *lens, int64_t n,
                                int64_t T, int32_t K, uint64_t *raw, uint64_t cap, unsigned long long *counters,
                                cudaStream_t s);
-// EmbedJoin+ (ej_plus.cu): the suffix set of every string (record q = i*S + k)
-// and the candidate pairs from the sorted record-pair matches.
-cudaError_t launch_suffix_lengths(const int32_t *lens, int64_t n, int32_t S, int32_t delta, uint32_t *sub_len,
-                                  int32_t *whole_len, cudaStream_t s);
-cudaError_t launch_suffix_copy(const uint8_t *bytes, const int64_t *offsets, int64_t n, int32_t S, int32_t delta,
-                               const uint64_t *sub_off, uint8_t *out, cudaStream_t s);
+// EmbedJoin+ (ej_plus.cu): the suffixes of every string as records (record q = i*S
+// + k) and the candidate pairs from the sorted record-pair matches.
+cudaError_t launch_suffix_records(const int32_t *lens, const int64_t *offsets, int64_t n, int32_t S, int32_t delta, int B,
+                                  int32_t *sub_len, uint32_t *counts, int64_t *start, int32_t *whole_len, cudaStream_t s);
 cudaError_t launch_plus_runs(const uint64_t *sorted, int64_t nraw, int32_t S, int32_t T, uint64_t *out,
                              uint64_t cap, unsigned long long *count, unsigned long long *same, cudaStream_t s);
 // Buckets by hashing (ej_join): per-table signature sets of H slots

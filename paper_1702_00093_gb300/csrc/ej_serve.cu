@@ -291,9 +291,8 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     SV(cudaMemsetAsync(sl.queue.p, 0, (size_t)nc * 8, s));
     SV(cudaMemsetAsync(sl.tickets.p, 0, (size_t)nc * SM_TICKETS * 4, s));
     // pack, walk and sign the queries with the index's tables
-    SV(launch_validate(qbytes, qoffs, Q, total, x.set.code_map, P<int32_t>(sl.qlens), derr,
+    SV(launch_validate(qbytes, qoffs, Q, total, x.set.B, P<int32_t>(sl.qlens), P<uint32_t>(sl.ccnt), derr,
                        (unsigned long long *)(derr + 2), s));
-    SV(launch_chunk_counts(P<int32_t>(sl.qlens), Q, x.set.B, P<uint32_t>(sl.ccnt), s));
     SV(exclusive_scan_u32(P<uint32_t>(sl.ccnt), P<uint64_t>(sl.qpofs), Q + 1, nullptr, sl.scan.p, s));
     SV(launch_pack(qbytes, qoffs, P<int32_t>(sl.qlens), Q, total, x.set.code_map, x.set.B, P<uint64_t>(sl.qpofs),
                    P<uint4>(sl.qpacked), derr, s));
