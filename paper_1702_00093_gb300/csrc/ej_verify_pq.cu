@@ -35,7 +35,8 @@
 //
 // What bounds it: 32-bit integer instructions, 10 W + about 8 per column. With
 // many pairs (5.4M candidates of 20000 reads of 5000 bases at K = 250) the launch
-// takes 21.7 ms at three warps per sub-partition (23.8 at two, 33.2 at one),
+// takes 20.5 ms at three warps per sub-partition (23.8 at two, 33.2 at one when
+// slots refilled one by one, 21.7 then at three),
 // against 28.2 ms for the block-aligned window with a test per column that this
 // form replaces; with few (about 13000, K = 250) it is set by the columns of its
 // longest pairs on one warp per sub-partition, 0.38 against 0.50 ms, and 0.25
@@ -280,8 +281,15 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
             if (lane == 0) warp_err((uint32_t)DERR_TIMEOUT);
             break;
         }
-        // refill free slots (both lanes of a slot agree on `have` and `exhausted`)
-        while (true) {
+        // refill free slots (both lanes of a slot agree on `have` and `exhausted`),
+        // several at a time: a refill takes the whole warp through the loads and the
+        // W + 1 match words of its pairs however few they are, and pairs that start
+        // together mostly end together (956000 text-like pairs, W = 4: one slot at a
+        // time 3.94 ms, four 2.82, eight 2.72; 5.7M DNA pairs, W = 8: 21.6, four 20.5)
+        constexpr int REFILL = B == 8 ? 8 : 4;
+        const unsigned idle = __ballot_sync(FULL, !have && !exhausted && !rev);
+        const bool refill = idle && (__popc(idle) >= REFILL || !__any_sync(FULL, have));
+        while (refill) {
             const bool need = !have && !exhausted;
             const unsigned nb = __ballot_sync(FULL, need && !rev);
             if (nb == 0u) break;
@@ -397,7 +405,7 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         }
         T += 32 - __popc(tacc);
         j0 += 32;
-        if ((iters & 1) == 0) {   // the joint bound
+        if ((iters & 1) == 0) {   // the joint bound (every chunk: 2.92 against 2.72 ms on text, W = 4)
             const int32_t lb = T + diag_min<W>(P, M, s_tab);
             const int32_t lb_other = __shfl_xor_sync(FULL, lb, 1);
             if (have && j0 < ncols && lb + lb_other > kp) rejected = true;
