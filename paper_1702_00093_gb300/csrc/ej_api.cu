@@ -973,7 +973,7 @@ int back_finish(ej_ctx *ctx, const Plan &pl, const ej_params *p, const unsigned 
     unsigned long long *cnt = (unsigned long long *)ctx->bufs[B_JCOUNT].p;
     const uint64_t *sorted = app;
     if (cntout <= small_sort_max()) {
-        CK(launch_small_sort(app, cnt + 3, (uint64_t)cntout, s));
+        CK(launch_small_sort(app, cnt + 3, (uint64_t)cntout, n, s));
     } else {
         const int nb = bits_for((uint64_t)(n - 1));
         int shifts[16], np = 0;
@@ -1573,7 +1573,7 @@ int batch_issue(ej_batch *b, cudaStream_t s) {
         const cudaStream_t js = j.side;
         unsigned long long *cnt = (unsigned long long *)j.sub->bufs[B_JCOUNT].p;
         if ((j.seg >= 0 && cudaStreamWaitEvent(js, b->fork, 0) != cudaSuccess) ||
-            launch_small_sort((uint64_t *)j.sub->bufs[B_APP].p, cnt + 3, (uint64_t)small_sort_max(), js) != cudaSuccess ||
+            launch_small_sort((uint64_t *)j.sub->bufs[B_APP].p, cnt + 3, (uint64_t)small_sort_max(), j.pl.st.n, js) != cudaSuccess ||
             cudaMemcpyAsync(b->h_stat + 16 * k, cnt, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, js) !=
                 cudaSuccess ||
             cudaMemcpyAsync(b->h_stat + 16 * k + 8, j.sub->bufs[B_DERR].p, sizeof(uint32_t), cudaMemcpyDeviceToHost,

@@ -364,7 +364,9 @@ constexpr int SX_MAX_WORDS = 12;
 SxBand sx_band(int32_t K);
 size_t sx_smem_bytes(int W, uint32_t alpha);
 int small_sort_max();
-cudaError_t launch_small_sort(uint64_t *a, const unsigned long long *count_dev, uint64_t n_cap, cudaStream_t s);
+// Pairs of strings below n_str, their number on the device (nothing if above n_cap).
+cudaError_t launch_small_sort(uint64_t *a, const unsigned long long *count_dev, uint64_t n_cap, int64_t n_str,
+                              cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Verification (ej_verify.cu)
