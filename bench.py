@@ -55,14 +55,14 @@ METRIC = "verified pairs/s (candidate pairs verified per second of whole-join wa
 # GB300: 152 SMs; the derived figure assumes 64 integer ALU lanes per SM per clock
 # at the maximum SM clock (kept beside the measured rate for context)
 SMS, ALU_LANES_PER_SM, MAX_SM_MHZ = 152, 64, 2070.0
-INT_OPS_PER_WORD_COLUMN = 26   # 32-bit ops of one 64-bit word of the bit-parallel step
+INT_OPS_PER_WORD_COLUMN = 20   # 32-bit ops of 64 rows of the bit-parallel step (ten per 32-bit word)
 HBM_FALLBACK_GBS = 6800.0
 VERIFY_SOURCE = os.path.join(ROOT, "paper_1702_00093_gb300", "csrc", "ej_verify_pq.cu")
 # DRAM bytes per verify launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture of the long-DNA workload: "merged" = the batch's merged launch,
 # "join" = mean over the K=50/150/250 launches of ej_join; valid only while the
 # verify source is the one that was captured
-VERIFY_TRAFFIC = {"source_sha256_prefix": "de1e03ec8e06edd5", "bytes_per_launch": {"merged": 13802496, "join": None}}
+VERIFY_TRAFFIC = {"source_sha256_prefix": "def08a6506c5d4ca", "bytes_per_launch": {"merged": 13691904, "join": None}}
 RECALL_SAMPLES = os.path.join(ROOT, "oracle", "recall_samples.json")
 
 
@@ -459,7 +459,7 @@ def stage_rooflines(ss, params, jstats, steps, hbm_gbs, hbm_src) -> dict:
         out[k] = {"bound": "hbm", "achieved": gbs, "peak": hbm_gbs, "unit": "GB/s", "frac": gbs / hbm_gbs,
                   "bytes_per_step": by, "ms_per_step": ms}
     out["peak_source"] = hbm_src + " (of measured)" if hbm_src.startswith("measured") else hbm_src
-    out["kernels"] = {"pack": "validate_offsets_kernel, chunk counts, scan, pack_kernel",
+    out["kernels"] = {"pack": "validate_offsets_kernel, scan, pack2_kernel or pack8_kernel",
                       "walk": "embed_sign_kernel (fused CGK walk + signatures; bound by instruction issue, "
                               "not by HBM: see profiles/embed_sign_long_dna.md)",
                       "buckets": "bucket_table_kernel (shared-memory tables) or bucket_insert/emit (global) or "
@@ -478,7 +478,8 @@ def verify_roofline(word_cols, ms, launches, int_peak, kernel, measured_in, traf
             "launches": launches, "avg_launch_ms": ms / max(launches, 1),
             "ops_per_word_column": INT_OPS_PER_WORD_COLUMN, "word_columns": word_cols,
             "word_columns_basis": ("columns advanced x 64-bit words of each pair's band (K_lo + K_hi + 1 <= K + 1 "
-                                   "diagonals for the persistent verifier, 2K + 1 for the others)"),
+                                   "diagonals for the persistent and shared-string verifiers, 2K + 1 for the "
+                                   "others)"),
             "measured_in": measured_in,
             "peak_basis": (int_peak["basis"] if int_peak else "derived: 152 SMs x 64 lanes/clock x 2070 MHz"),
             "derived_alu_peak": derived / 1e12}
@@ -776,8 +777,9 @@ def run_join_workload(ej, ctx, ss, params, dev, stream, flush, world, clk, steps
         n_verify = sum(1 for _, _, s in jstats if s["n_candidates"] > 0)
         res["join_roofline"] = verify_roofline(
             word_cols, verify_ms, n_verify, int_peak,
-            "the verifier of ej_join, one launch per join (persistent verify_pq_kernel for mean string length "
-            ">= 2048, else grid-strided verify_bd_kernel)",
+            "the verifier of ej_join, one per join (persistent verify_pq_kernel, or, for more than four symbols at "
+            "mean lengths below 2048 and for dense signatures, shared-string verify_sx_kernel and the pairs it "
+            "hands on)",
             "the ej_join pass (CUDA events around each verify launch, its stream)", verify_traffic("join"))
         res["stage_roofline"] = stage_rooflines(ss, params, jstats, join_steps, hbm[0], hbm[1])
         per_k = {}
@@ -878,7 +880,9 @@ def high_recall_summary(ej, ctx, ss, params, dev, stream, flush, world, clk, int
                           paths={"batch", "join", "eager"}, plain_steps=0, e2e_steps=0, autotune=False,
                           batch_eager=False, int_peak=int_peak, hbm=hbm, timed_windows=[])
     rec = cluster_recall(ej, ctx, ss, hp, r["result_pairs"], dev, stream)
-    roof = r.get("merged_roofline") or r.get("join_roofline")
+    # from the ej_join pass: the largest join's candidates are dense enough for the
+    # shared-string verifier, so the batch's merged launch holds the others only
+    roof = r.get("join_roofline")
     if roof is not None:
         # the stored ncu DRAM bytes belong to the headline's launch, not to this one
         roof = dict(roof, traffic=None)

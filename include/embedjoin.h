@@ -122,8 +122,8 @@ typedef struct {
                                 verification, counted algorithmically) */
     uint64_t verify_word_columns; /* 64-bit words of the band the verifier runs
                                 times the columns it actually advanced (early
-                                exit included): the persistent verifier runs the
-                                diagonals a cost-K alignment can use given the
+                                exit included): the persistent and the shared-
+                                string verifier run the diagonals a cost-K alignment can use given the
                                 pair's length difference d, K_lo + K_hi + 1 <= K + 1
                                 (K_lo = floor((K-d)/2), K_hi = floor((K+d)/2)),
                                 ceil((K_lo + K_hi + 1)/64) words; the others run
