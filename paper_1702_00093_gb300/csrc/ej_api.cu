@@ -642,7 +642,7 @@ int verify_dev(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *
     // the persistent verifier unless a tiling was asked for or its window does not
     // fit: its band is half of Ukkonen's and its slots refill (against the grid-
     // strided one: 5000-base reads, K = 150, 0.85 -> 0.26 ms; 900000 text-like
-    // candidates, K = 100, 9.7 -> 3.9 ms)
+    // candidates, K = 100, 9.7 -> 2.7 ms)
     const int pq_threads = ctx->vG > 0 ? 0 : pq_threads_for(pq_words(p->K), p->alphabet_size);
     if (pq_threads > 0) {
         CK(cudaMemsetAsync(tickets, 0, SM_TICKETS * sizeof(unsigned int), s));
