@@ -212,6 +212,9 @@ pack2_kernel(const uint8_t *__restrict__ bytes, const int64_t *__restrict__ offs
 }
 
 // 16 bytes from byte offset bs / 8 of word WO on of chunks c0[h], c0[h + 1], looked up.
+// A byte outside the alphabet is noted in `bad` and stored as code 0: a search and a
+// batch replay walk and verify the codes before the host reads the error word, and
+// both index their tables with them.
 __device__ __forceinline__ uint4 pack16(const uint32_t (&u)[5], uint32_t bs, const uint8_t *s_map, uint32_t &bad) {
     uint32_t out[4];
 #pragma unroll
@@ -221,7 +224,9 @@ __device__ __forceinline__ uint4 pack16(const uint32_t (&u)[5], uint32_t bs, con
 #pragma unroll
         for (int j = 0; j < 4; j++) c[j] = s_map[__byte_perm(w, 0u, 0x4440 | j)];
         out[q] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
-        bad |= ((out[q] & 0x7F7F7F7Fu) + 0x01010101u) & out[q] & 0x80808080u;   // a byte of 255
+        const uint32_t none = ((out[q] & 0x7F7F7F7Fu) + 0x01010101u) & out[q] & 0x80808080u;   // bytes of 255
+        bad |= none;
+        out[q] &= ~((none >> 7) * 255u);
     }
     return make_uint4(out[0], out[1], out[2], out[3]);
 }
