@@ -187,8 +187,9 @@ pack2_kernel(const uint8_t *__restrict__ bytes, const int64_t *__restrict__ offs
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
                         const uint32_t c = s_map[__byte_perm(w[q], 0u, 0x4440 | j)];
-                        bad |= c & 0x80u;   // 255: none (codes are below 4)
-                        cw |= (c & 3u) << (24 + 2 * j);
+                        const bool none = c & 0x80u;   // 255 (codes are below 4): code 0, a code of every alphabet
+                        bad |= none;
+                        cw |= (none ? 0u : c) << (24 + 2 * j);
                     }
                     out[q] = cw;
                 }

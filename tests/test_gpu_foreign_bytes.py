@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 DEV = "cuda:0"
-ALPHABETS = [(synth.PROTEIN, b"J"), (synth.TEXT, b"~"), (b"ACGTN", bytes([255]))]
+ALPHABETS = [(synth.PROTEIN, b"J"), (synth.TEXT, b"~"), (b"ACGTN", bytes([255])),
+             (b"ACGT", b"N"), (bytes([0, 1, 64]), bytes([2])), (bytes([0, 64]), bytes([1]))]   # packed in 2 bits
 
 
 @pytest.fixture(scope="module")
