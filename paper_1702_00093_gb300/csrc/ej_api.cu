@@ -265,7 +265,7 @@ int make_plan(ej_ctx *ctx, const ej_strings *S, const ej_params *p, bool need_ls
     const int64_t chunk_bound = (total * pl->B + 127) / 128 + n + 1;
     CKS(ensure_t(ctx, B_PACKED, (size_t)chunk_bound, &packed));
     CK(launch_validate(pl->st.bytes, pl->st.offsets, n, total, pl->B, pl->lens, ccnt, derr, dmax, s));
-    CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, stmp, s));
+    CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, stmp, s, derr));
     CK(launch_pack(pl->st.bytes, pl->st.offsets, pl->lens, n, total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl->B,
                    pofs, packed, derr, s));
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[7], s));
@@ -313,7 +313,7 @@ int plan_device(ej_ctx *ctx, const Plan &pl, cudaStream_t s) {
     unsigned long long *dmax = (unsigned long long *)(derr + 2);
     uint32_t *ccnt = (uint32_t *)ctx->bufs[B_CHUNK_CNT].p;
     CK(launch_validate(pl.st.bytes, pl.st.offsets, n, pl.st.total, pl.B, pl.lens, ccnt, derr, dmax, s));
-    CK(exclusive_scan_u32(ccnt, (uint64_t *)pl.pofs, n + 1, nullptr, ctx->bufs[B_SCAN_TMP3].p, s));
+    CK(exclusive_scan_u32(ccnt, (uint64_t *)pl.pofs, n + 1, nullptr, ctx->bufs[B_SCAN_TMP3].p, s, derr));
     CK(launch_pack(pl.st.bytes, pl.st.offsets, pl.lens, n, pl.st.total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl.B,
                    pl.pofs, (uint4 *)pl.packed, derr, s));
     return EJ_OK;
@@ -2047,11 +2047,11 @@ int ej_join_plus(ej_ctx *ctx, const ej_strings *S, const ej_params *p, int32_t d
     sp.out_len = pl.out_len;
     sp.L = pl.L;
     int st = upload_alphabet(sub, &sp, s);
-    uint32_t *counts = nullptr;
+    uint32_t *counts = nullptr, *derr = nullptr;
     uint64_t *spofs = nullptr;
     uint4 *spacked = nullptr;
     void *stmp0 = nullptr;
-    if (st == EJ_OK) st = ensure_t(sub, B_DERR, 8, (uint32_t **)&stmp0);
+    if (st == EJ_OK) st = ensure_t(sub, B_DERR, 8, &derr);
     if (st == EJ_OK) st = ensure_t(sub, B_LENS, (size_t)nq, &spl.lens);
     if (st == EJ_OK) st = ensure_t(sub, B_CHUNK_CNT, (size_t)nq + 1, &counts);
     if (st == EJ_OK) st = ensure_t(sub, B_POFS, (size_t)nq + 2, &spofs);
@@ -2060,10 +2060,11 @@ int ej_join_plus(ej_ctx *ctx, const ej_strings *S, const ej_params *p, int32_t d
     const int64_t chunk_bound = nsub * ((pl.st.total * pl.B + 127) / 128 + n) + 1;
     if (st == EJ_OK) st = ensure_t(sub, B_PACKED, (size_t)chunk_bound, &spacked);
     if (st != EJ_OK) return sub_fail(st);
+    CK(cudaMemsetAsync(derr, 0, 4, s));
     CK(launch_suffix_records(pl.lens, pl.st.offsets, n, nsub, delta, pl.B, spl.lens, counts, start, whole, s));
     CK(exclusive_scan_u32(counts, spofs, nq + 1, nullptr, stmp0, s));
     CK(launch_pack(pl.st.bytes, start, spl.lens, nq, pl.st.total, (const uint8_t *)sub->bufs[B_CODEMAP].p, pl.B, spofs,
-                   spacked, (uint32_t *)sub->bufs[B_DERR].p, s));
+                   spacked, derr, s));
     spl.packed = spacked;
     spl.pofs = spofs;
     uint64_t *keys = nullptr;
@@ -2074,14 +2075,12 @@ int ej_join_plus(ej_ctx *ctx, const ej_strings *S, const ej_params *p, int32_t d
     // buckets of the suffix records, matches filtered by the whole strings' lengths
     const uint64_t H = bucket_slots_per_table(nq);
     uint64_t *bkeys = nullptr;
-    uint32_t *bheads = nullptr, *bnext = nullptr, *derr = nullptr;
+    uint32_t *bheads = nullptr, *bnext = nullptr;
     unsigned long long *cnt = nullptr;
     CKS(ensure_t(sub, B_BKEYS, (size_t)(H * TT), &bkeys));
     CKS(ensure_t(sub, B_BHEADS, (size_t)(H * TT), &bheads));
     CKS(ensure_t(sub, B_BNEXT, (size_t)(nq * TT), &bnext));
-    CKS(ensure_t(sub, B_DERR, 8, &derr));
     CKS(ensure_t(sub, B_JCOUNT, JCOUNT_LEN, &cnt));
-    CK(cudaMemsetAsync(derr, 0, 4, s));
     CK(cudaMemsetAsync(bkeys, 0xFF, H * TT * sizeof(uint64_t), s));
     CK(cudaMemsetAsync(bheads, 0xFF, H * TT * sizeof(uint32_t), s));
     CK(launch_bucket_insert(keys, nq, TT, H, bkeys, bheads, bnext, derr, s));

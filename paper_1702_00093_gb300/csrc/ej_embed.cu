@@ -96,6 +96,7 @@ pack2_kernel(const uint8_t *__restrict__ bytes, const int64_t *__restrict__ offs
              const int32_t *__restrict__ lens, int64_t n, int64_t total,
              const uint8_t *__restrict__ code_map, const uint64_t *__restrict__ pofs,
              uint4 *__restrict__ packed, uint32_t *__restrict__ err) {
+    if (*err & DERR_OFFSETS) return;   // the strings do not fit the buffer
     __shared__ uint8_t s_map[256];
     __shared__ uint32_t s_sym[4];     // the symbol of each code (0x100: none)
     __shared__ uint32_t s_tab[4];     // code_lo, code_hi, sym_lo, sym_hi of the PackMap
@@ -253,6 +254,7 @@ pack8_kernel(const uint8_t *__restrict__ bytes, const int64_t *__restrict__ offs
              const int32_t *__restrict__ lens, int64_t n, int64_t total,
              const uint8_t *__restrict__ code_map, const uint64_t *__restrict__ pofs,
              uint4 *__restrict__ packed, uint32_t *__restrict__ err) {
+    if (*err & DERR_OFFSETS) return;   // the strings do not fit the buffer
     __shared__ uint8_t s_map[256];
     __shared__ uint32_t s_fill;     // four times the symbol of code 0
     for (int t = threadIdx.x; t < 256; t += blockDim.x) {

@@ -105,7 +105,11 @@ enum : uint32_t {
 // ---------------------------------------------------------------------------
 
 // Validation + lengths: lens[i] = offsets[i+1]-offsets[i], counts[i] = its chunks
-// of B-bit codes (counts[n] = 0); err |= DERR_*; *max_len = max length.
+// of B-bit codes (counts[n] = 0); err |= DERR_*; *max_len = max length. Every string
+// is checked alone, so offsets that go up and down leave lengths that are each at
+// most total_cap and together more: the scan of the counts and the packing take err
+// and then place every string at chunk 0 and write nothing, so that what runs before
+// the host reads err stays inside a buffer sized for total_cap bytes.
 cudaError_t launch_validate(const uint8_t *bytes, const int64_t *offsets, int64_t n, int64_t total_cap,
                             int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
                             cudaStream_t s);
@@ -120,7 +124,7 @@ cudaError_t launch_positions(uint64_t seed, uint32_t r, uint32_t m, uint32_t z, 
                              const uint32_t *pos_inject, uint32_t *pos, cudaStream_t s);
 
 // Pack bytes -> codes; bytes outside the alphabet set DERR_SYMBOL (some code of the
-// alphabet is stored).
+// alphabet is stored). Nothing is packed with DERR_OFFSETS in *err.
 // total: bytes in the array (every validated string lies inside [0, total)).
 cudaError_t launch_pack(const uint8_t *bytes, const int64_t *offsets, const int32_t *lens, int64_t n, int64_t total,
                         const uint8_t *code_map, int B, const uint64_t *pofs, uint4 *packed,
@@ -190,8 +194,10 @@ cudaError_t launch_remap_pairs(const uint64_t *pairs, int64_t cnt, const int32_t
 size_t scan_temp_bytes(int64_t n);
 cudaError_t exclusive_scan_u8(const uint8_t *in, uint64_t *out, int64_t n, uint64_t *total_dev,
                               void *temp, cudaStream_t s);
+// err (u32, may be null): error word of the strings the values were counted for;
+// with DERR_OFFSETS in it every value counts as 0.
 cudaError_t exclusive_scan_u32(const uint32_t *in, uint64_t *out, int64_t n, uint64_t *total_dev,
-                               void *temp, cudaStream_t s);
+                               void *temp, cudaStream_t s, const uint32_t *err = nullptr);
 
 // Stable LSD radix sort of `nseg` independent segments of `seg_len` records
 // each (segment k occupies [k*seg_len, (k+1)*seg_len)), by 8-bit digits at the

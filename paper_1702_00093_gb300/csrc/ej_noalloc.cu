@@ -130,7 +130,7 @@ extern "C" int ej_verify_noalloc(const ej_strings *S, const ej_params *p, const 
     NA_CK(cudaMemcpyAsync(d_map, map, 256, cudaMemcpyHostToDevice, s));
     unsigned long long *dmax = (unsigned long long *)(err + 2);
     NA_CK(launch_validate(S->bytes, S->offsets, n, total, B, lens, ccnt, err, dmax, s));
-    NA_CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, scan_a, s));
+    NA_CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, scan_a, s, err));
     NA_CK(launch_pack(S->bytes, S->offsets, lens, n, total, d_map, B, pofs, packed, err, s));
     uint64_t h[2] = {0, 0};
     NA_CK(cudaMemcpyAsync(h, err, 16, cudaMemcpyDeviceToHost, s));

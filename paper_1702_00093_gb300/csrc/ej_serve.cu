@@ -293,7 +293,8 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     // pack, walk and sign the queries with the index's tables
     SV(launch_validate(qbytes, qoffs, Q, total, x.set.B, P<int32_t>(sl.qlens), P<uint32_t>(sl.ccnt), derr,
                        (unsigned long long *)(derr + 2), s));
-    SV(exclusive_scan_u32(P<uint32_t>(sl.ccnt), P<uint64_t>(sl.qpofs), Q + 1, nullptr, sl.scan.p, s));
+    SV(exclusive_scan_u32(P<uint32_t>(sl.ccnt), P<uint64_t>(sl.qpofs), Q + 1, nullptr, sl.scan.p, s,
+                          derr));
     SV(launch_pack(qbytes, qoffs, P<int32_t>(sl.qlens), Q, total, x.set.code_map, x.set.B, P<uint64_t>(sl.qpofs),
                    P<uint4>(sl.qpacked), derr, s));
     SV(launch_embed_sign(P<uint4>(sl.qpacked), P<uint64_t>(sl.qpofs), P<int32_t>(sl.qlens), Q, x.p.r, x.p.m, x.p.z,

@@ -47,10 +47,18 @@ __device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t *total,
     return res;
 }
 
+// Every value counts as 0: the values are the chunks of strings whose offsets failed
+// the validation (err, may be null).
+__device__ __forceinline__ bool scan_voided(const uint32_t *__restrict__ err) {
+    return err && (*err & DERR_OFFSETS);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(SCAN_THREADS)
-scan_reduce_kernel(const T *__restrict__ in, int64_t n, uint64_t *__restrict__ block_sums) {
+scan_reduce_kernel(const T *__restrict__ in, int64_t n, uint64_t *__restrict__ block_sums,
+                   const uint32_t *__restrict__ err) {
     __shared__ uint64_t s_warp[SCAN_THREADS / 32 + 1];
+    if (scan_voided(err)) n = 0;
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK;
     uint64_t sum = 0;
 #pragma unroll
@@ -97,15 +105,16 @@ scan_sums_kernel(uint64_t *__restrict__ sums, int64_t nb, uint64_t *__restrict__
 template <typename T>
 __global__ void __launch_bounds__(SCAN_THREADS)
 scan_apply_kernel(const T *__restrict__ in, uint64_t *__restrict__ out, int64_t n,
-                  const uint64_t *__restrict__ block_offs) {
+                  const uint64_t *__restrict__ block_offs, const uint32_t *__restrict__ err) {
     __shared__ uint64_t s_warp[SCAN_THREADS / 32 + 1];
+    const bool voided = scan_voided(err);
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
     uint64_t v[SCAN_ITEMS];
     uint64_t local = 0;
 #pragma unroll
     for (int it = 0; it < SCAN_ITEMS; it++) {
         int64_t i = base + it;
-        v[it] = i < n ? (uint64_t)in[i] : 0;
+        v[it] = i < n && !voided ? (uint64_t)in[i] : 0;
         local += v[it];
     }
     uint64_t tot;
@@ -123,15 +132,17 @@ scan_apply_kernel(const T *__restrict__ in, uint64_t *__restrict__ out, int64_t 
 constexpr int64_t SCAN_ONE = 4 * SCAN_CHUNK;
 template <typename T>
 __global__ void __launch_bounds__(SCAN_THREADS)
-scan_one_kernel(const T *__restrict__ in, uint64_t *__restrict__ out, int64_t n, uint64_t *__restrict__ total_dev) {
+scan_one_kernel(const T *__restrict__ in, uint64_t *__restrict__ out, int64_t n, uint64_t *__restrict__ total_dev,
+                const uint32_t *__restrict__ err) {
     __shared__ uint64_t s_warp[SCAN_THREADS / 32 + 1];
+    const bool voided = scan_voided(err);
     uint64_t carry = 0;
     for (int64_t base = 0; base < n; base += SCAN_CHUNK) {
         const int64_t first = base + (int64_t)threadIdx.x * SCAN_ITEMS;
         uint64_t v[SCAN_ITEMS], local = 0, tot;
 #pragma unroll
         for (int it = 0; it < SCAN_ITEMS; it++) {
-            v[it] = first + it < n ? (uint64_t)in[first + it] : 0;
+            v[it] = first + it < n && !voided ? (uint64_t)in[first + it] : 0;
             local += v[it];
         }
         uint64_t run = carry + block_excl_scan(local, &tot, s_warp);
@@ -147,17 +158,17 @@ scan_one_kernel(const T *__restrict__ in, uint64_t *__restrict__ out, int64_t n,
 
 template <typename T>
 static cudaError_t exclusive_scan(const T *in, uint64_t *out, int64_t n, uint64_t *total_dev,
-                                  void *temp, cudaStream_t s) {
+                                  void *temp, cudaStream_t s, const uint32_t *err = nullptr) {
     uint64_t *sums = (uint64_t *)temp;
     if (n <= SCAN_ONE) {
-        scan_one_kernel<T><<<1, SCAN_THREADS, 0, s>>>(in, out, n, total_dev);
+        scan_one_kernel<T><<<1, SCAN_THREADS, 0, s>>>(in, out, n, total_dev, err);
         note_launches(1);
         return cudaGetLastError();
     }
     const int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-    if (nb > 0) scan_reduce_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums);
+    if (nb > 0) scan_reduce_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums, err);
     scan_sums_kernel<<<1, SCAN_THREADS, 0, s>>>(sums, nb, total_dev);
-    if (nb > 0) scan_apply_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums);
+    if (nb > 0) scan_apply_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums, err);
     note_launches(nb > 0 ? 3 : 1);
     return cudaGetLastError();
 }
@@ -167,8 +178,8 @@ cudaError_t exclusive_scan_u8(const uint8_t *in, uint64_t *out, int64_t n, uint6
     return exclusive_scan<uint8_t>(in, out, n, total_dev, temp, s);
 }
 cudaError_t exclusive_scan_u32(const uint32_t *in, uint64_t *out, int64_t n, uint64_t *total_dev,
-                               void *temp, cudaStream_t s) {
-    return exclusive_scan<uint32_t>(in, out, n, total_dev, temp, s);
+                               void *temp, cudaStream_t s, const uint32_t *err) {
+    return exclusive_scan<uint32_t>(in, out, n, total_dev, temp, s, err);
 }
 
 // ---------------------------------------------------------------------------
