@@ -264,7 +264,7 @@ int make_plan(ej_ctx *ctx, const ej_strings *S, const ej_params *p, bool need_ls
     CKS(ensure(ctx, B_SCAN_TMP3, scan_temp_bytes(n + 1), &stmp));
     const int64_t chunk_bound = (total * pl->B + 127) / 128 + n + 1;
     CKS(ensure_t(ctx, B_PACKED, (size_t)chunk_bound, &packed));
-    CK(launch_validate(pl->st.bytes, pl->st.offsets, n, total, pl->B, pl->lens, ccnt, derr, dmax, s));
+    CK(launch_validate(pl->st.bytes, pl->st.offsets, n, total, ANY_LEN, pl->B, pl->lens, ccnt, derr, dmax, s));
     CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, stmp, s, derr));
     CK(launch_pack(pl->st.bytes, pl->st.offsets, pl->lens, n, total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl->B,
                    pofs, packed, derr, s));
@@ -312,7 +312,7 @@ int plan_device(ej_ctx *ctx, const Plan &pl, cudaStream_t s) {
     CK(cudaMemsetAsync(derr, 0, 4 * sizeof(uint32_t), s));
     unsigned long long *dmax = (unsigned long long *)(derr + 2);
     uint32_t *ccnt = (uint32_t *)ctx->bufs[B_CHUNK_CNT].p;
-    CK(launch_validate(pl.st.bytes, pl.st.offsets, n, pl.st.total, pl.B, pl.lens, ccnt, derr, dmax, s));
+    CK(launch_validate(pl.st.bytes, pl.st.offsets, n, pl.st.total, pl.max_len, pl.B, pl.lens, ccnt, derr, dmax, s));
     CK(exclusive_scan_u32(ccnt, (uint64_t *)pl.pofs, n + 1, nullptr, ctx->bufs[B_SCAN_TMP3].p, s, derr));
     CK(launch_pack(pl.st.bytes, pl.st.offsets, pl.lens, n, pl.st.total, (const uint8_t *)ctx->bufs[B_CODEMAP].p, pl.B,
                    pl.pofs, (uint4 *)pl.packed, derr, s));

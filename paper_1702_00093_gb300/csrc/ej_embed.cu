@@ -12,8 +12,12 @@ namespace ej {
 
 // total_cap bounds offsets[n]: beyond it every length is reported as 0 (and
 // DERR_OFFSETS set), so that buffers sized for total_cap bytes are never overrun.
+// A string longer than len_cap counts to *max_len and is then taken as empty: a
+// batch's replay runs with tables sized for its plan's longest string (the shared
+// match masks of the verifier with four and more lanes per pair) before the host
+// compares *max_len with it.
 __global__ void validate_offsets_kernel(const int64_t *__restrict__ offsets, int64_t n, int64_t total_cap,
-                                        int B, int32_t *__restrict__ lens,
+                                        int64_t len_cap, int B, int32_t *__restrict__ lens,
                                         uint32_t *__restrict__ counts, uint32_t *__restrict__ err,
                                         unsigned long long *__restrict__ max_len) {
     unsigned long long local_max = 0;
@@ -28,9 +32,10 @@ __global__ void validate_offsets_kernel(const int64_t *__restrict__ offsets, int
             local_err |= DERR_OFFSETS;
             len = 0;
         }
+        local_max = len > (int64_t)local_max ? (unsigned long long)len : local_max;
+        if (len > len_cap) len = 0;
         lens[i] = (int32_t)len;
         counts[i] = (uint32_t)chunks_for(len, B);
-        local_max = len > (int64_t)local_max ? (unsigned long long)len : local_max;
     }
     for (int o = 16; o > 0; o >>= 1) {
         unsigned long long v = __shfl_xor_sync(FULL, local_max, o);
@@ -44,12 +49,12 @@ __global__ void validate_offsets_kernel(const int64_t *__restrict__ offsets, int
 }
 
 cudaError_t launch_validate(const uint8_t *bytes, const int64_t *offsets, int64_t n, int64_t total_cap,
-                            int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
+                            int64_t len_cap, int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
                             cudaStream_t s) {
     if (n == 0) return cudaMemsetAsync(counts, 0, sizeof(uint32_t), s);
     int grid = (int)((n + 255) / 256);
     if (grid > 4096) grid = 4096;
-    validate_offsets_kernel<<<grid, 256, 0, s>>>(offsets, n, total_cap, B, lens, counts, err, max_len);
+    validate_offsets_kernel<<<grid, 256, 0, s>>>(offsets, n, total_cap, len_cap, B, lens, counts, err, max_len);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -105,13 +105,15 @@ enum : uint32_t {
 // ---------------------------------------------------------------------------
 
 // Validation + lengths: lens[i] = offsets[i+1]-offsets[i], counts[i] = its chunks
-// of B-bit codes (counts[n] = 0); err |= DERR_*; *max_len = max length. Every string
+// of B-bit codes (counts[n] = 0); err |= DERR_*; *max_len = max length; strings longer
+// than len_cap (at most 2^31 - 1) are then taken as empty. Every string
 // is checked alone, so offsets that go up and down leave lengths that are each at
 // most total_cap and together more: the scan of the counts and the packing take err
 // and then place every string at chunk 0 and write nothing, so that what runs before
 // the host reads err stays inside a buffer sized for total_cap bytes.
+constexpr int64_t ANY_LEN = 0x7fffffff;
 cudaError_t launch_validate(const uint8_t *bytes, const int64_t *offsets, int64_t n, int64_t total_cap,
-                            int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
+                            int64_t len_cap, int B, int32_t *lens, uint32_t *counts, uint32_t *err, unsigned long long *max_len,
                             cudaStream_t s);
 
 // Random-bit table [r][out_len][words]: bit c of row (l, j) = pi_j^l(alphabet[c]).

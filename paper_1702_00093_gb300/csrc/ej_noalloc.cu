@@ -129,7 +129,7 @@ extern "C" int ej_verify_noalloc(const ej_strings *S, const ej_params *p, const 
     NA_CK(cudaMemsetAsync(err, 0, 64, s));
     NA_CK(cudaMemcpyAsync(d_map, map, 256, cudaMemcpyHostToDevice, s));
     unsigned long long *dmax = (unsigned long long *)(err + 2);
-    NA_CK(launch_validate(S->bytes, S->offsets, n, total, B, lens, ccnt, err, dmax, s));
+    NA_CK(launch_validate(S->bytes, S->offsets, n, total, ANY_LEN, B, lens, ccnt, err, dmax, s));
     NA_CK(exclusive_scan_u32(ccnt, pofs, n + 1, nullptr, scan_a, s, err));
     NA_CK(launch_pack(S->bytes, S->offsets, lens, n, total, d_map, B, pofs, packed, err, s));
     uint64_t h[2] = {0, 0};

@@ -291,7 +291,7 @@ cudaError_t slot_launch(Slot &sl, const ej_index &x, const std::vector<Query> &q
     SV(cudaMemsetAsync(sl.queue.p, 0, (size_t)nc * 8, s));
     SV(cudaMemsetAsync(sl.tickets.p, 0, (size_t)nc * SM_TICKETS * 4, s));
     // pack, walk and sign the queries with the index's tables
-    SV(launch_validate(qbytes, qoffs, Q, total, x.set.B, P<int32_t>(sl.qlens), P<uint32_t>(sl.ccnt), derr,
+    SV(launch_validate(qbytes, qoffs, Q, total, ANY_LEN, x.set.B, P<int32_t>(sl.qlens), P<uint32_t>(sl.ccnt), derr,
                        (unsigned long long *)(derr + 2), s));
     SV(exclusive_scan_u32(P<uint32_t>(sl.ccnt), P<uint64_t>(sl.qpofs), Q + 1, nullptr, sl.scan.p, s,
                           derr));

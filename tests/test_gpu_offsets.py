@@ -103,3 +103,36 @@ def test_batch_replays_report_malformed_offsets(ej, alphabet, mode):
             b.close()
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8])
+@pytest.mark.parametrize("alphabet", [b"ACGT", synth.PROTEIN], ids=["dna", "protein"])
+def test_batch_replay_with_a_longer_string(ej, alphabet, lanes):
+    """The verifier of four and more lanes per pair sizes its match masks for the
+    planned longest string; a replay with a longer one reports it."""
+    ss = _set(alphabet, 60)
+    p = ej.Params(K=30, r=2, m=3, z=4, L=120, seed=4, alphabet=alphabet)
+    ctx, stream = ej.Context(0), torch.cuda.Stream()
+    try:
+        ctx.set_schedule(mode=2)
+        ctx.set_verify_config(lanes, 2 if lanes == 2 else 1)
+        with torch.cuda.stream(stream):
+            s = ej.Strings.from_set(ss, DEV)
+            b = ctx.batch(s, [p], stream=stream)
+            b.run(stream)
+            want, _ = b.result(0, device=DEV, stream=stream)
+            assert len(want) >= 30
+            merged = ss.offsets.copy()
+            merged[1:40] = merged[40]      # string 0 takes the bytes of the 39 after it
+            s.offsets.copy_(torch.from_numpy(merged))
+            b.run(stream)
+            with pytest.raises(ej.EJError) as e:
+                b.result(0, device=DEV, stream=stream)
+            assert e.value.status == ej.EJ_ERR_INVALID_ARG
+            s.offsets.copy_(torch.from_numpy(ss.offsets))
+            b.run(stream)
+            got, _ = b.result(0, device=DEV, stream=stream)
+            assert torch.equal(got, want)
+            b.close()
+    finally:
+        ctx.close()
