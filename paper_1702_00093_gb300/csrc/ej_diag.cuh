@@ -110,10 +110,34 @@ __device__ __forceinline__ void add_chain32<12>(uint32_t (&S)[12], const uint32_
         : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]));
 }
 template <>
+__device__ __forceinline__ void add_chain32<14>(uint32_t (&S)[14], const uint32_t (&A)[14], const uint32_t (&Bv)[14]) {
+    asm("add.cc.u32 %0, %14, %28;\n\taddc.cc.u32 %1, %15, %29;\n\taddc.cc.u32 %2, %16, %30;\n\taddc.cc.u32 %3, %17, %31;\n\taddc.cc.u32 %4, %18, %32;\n\taddc.cc.u32 %5, %19, %33;\n\taddc.cc.u32 %6, %20, %34;\n\taddc.cc.u32 %7, %21, %35;\n\taddc.cc.u32 %8, %22, %36;\n\taddc.cc.u32 %9, %23, %37;\n\taddc.cc.u32 %10, %24, %38;\n\taddc.cc.u32 %11, %25, %39;\n\taddc.cc.u32 %12, %26, %40;\n\taddc.u32 %13, %27, %41;"
+        : "=r"(S[0]), "=r"(S[1]), "=r"(S[2]), "=r"(S[3]), "=r"(S[4]), "=r"(S[5]), "=r"(S[6]), "=r"(S[7]), "=r"(S[8]), "=r"(S[9]), "=r"(S[10]), "=r"(S[11]), "=r"(S[12]), "=r"(S[13])
+        : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(A[12]), "r"(A[13]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]), "r"(Bv[12]), "r"(Bv[13]));
+}
+template <>
 __device__ __forceinline__ void add_chain32<16>(uint32_t (&S)[16], const uint32_t (&A)[16], const uint32_t (&Bv)[16]) {
     asm("add.cc.u32 %0, %16, %32;\n\taddc.cc.u32 %1, %17, %33;\n\taddc.cc.u32 %2, %18, %34;\n\taddc.cc.u32 %3, %19, %35;\n\taddc.cc.u32 %4, %20, %36;\n\taddc.cc.u32 %5, %21, %37;\n\taddc.cc.u32 %6, %22, %38;\n\taddc.cc.u32 %7, %23, %39;\n\taddc.cc.u32 %8, %24, %40;\n\taddc.cc.u32 %9, %25, %41;\n\taddc.cc.u32 %10, %26, %42;\n\taddc.cc.u32 %11, %27, %43;\n\taddc.cc.u32 %12, %28, %44;\n\taddc.cc.u32 %13, %29, %45;\n\taddc.cc.u32 %14, %30, %46;\n\taddc.u32 %15, %31, %47;"
         : "=r"(S[0]), "=r"(S[1]), "=r"(S[2]), "=r"(S[3]), "=r"(S[4]), "=r"(S[5]), "=r"(S[6]), "=r"(S[7]), "=r"(S[8]), "=r"(S[9]), "=r"(S[10]), "=r"(S[11]), "=r"(S[12]), "=r"(S[13]), "=r"(S[14]), "=r"(S[15])
         : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(A[12]), "r"(A[13]), "r"(A[14]), "r"(A[15]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]), "r"(Bv[12]), "r"(Bv[13]), "r"(Bv[14]), "r"(Bv[15]));
+}
+template <>
+__device__ __forceinline__ void add_chain32<18>(uint32_t (&S)[18], const uint32_t (&A)[18], const uint32_t (&Bv)[18]) {
+    asm("add.cc.u32 %0, %18, %36;\n\taddc.cc.u32 %1, %19, %37;\n\taddc.cc.u32 %2, %20, %38;\n\taddc.cc.u32 %3, %21, %39;\n\taddc.cc.u32 %4, %22, %40;\n\taddc.cc.u32 %5, %23, %41;\n\taddc.cc.u32 %6, %24, %42;\n\taddc.cc.u32 %7, %25, %43;\n\taddc.cc.u32 %8, %26, %44;\n\taddc.cc.u32 %9, %27, %45;\n\taddc.cc.u32 %10, %28, %46;\n\taddc.cc.u32 %11, %29, %47;\n\taddc.cc.u32 %12, %30, %48;\n\taddc.cc.u32 %13, %31, %49;\n\taddc.cc.u32 %14, %32, %50;\n\taddc.cc.u32 %15, %33, %51;\n\taddc.cc.u32 %16, %34, %52;\n\taddc.u32 %17, %35, %53;"
+        : "=r"(S[0]), "=r"(S[1]), "=r"(S[2]), "=r"(S[3]), "=r"(S[4]), "=r"(S[5]), "=r"(S[6]), "=r"(S[7]), "=r"(S[8]), "=r"(S[9]), "=r"(S[10]), "=r"(S[11]), "=r"(S[12]), "=r"(S[13]), "=r"(S[14]), "=r"(S[15]), "=r"(S[16]), "=r"(S[17])
+        : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(A[12]), "r"(A[13]), "r"(A[14]), "r"(A[15]), "r"(A[16]), "r"(A[17]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]), "r"(Bv[12]), "r"(Bv[13]), "r"(Bv[14]), "r"(Bv[15]), "r"(Bv[16]), "r"(Bv[17]));
+}
+template <>
+__device__ __forceinline__ void add_chain32<20>(uint32_t (&S)[20], const uint32_t (&A)[20], const uint32_t (&Bv)[20]) {
+    asm("add.cc.u32 %0, %20, %40;\n\taddc.cc.u32 %1, %21, %41;\n\taddc.cc.u32 %2, %22, %42;\n\taddc.cc.u32 %3, %23, %43;\n\taddc.cc.u32 %4, %24, %44;\n\taddc.cc.u32 %5, %25, %45;\n\taddc.cc.u32 %6, %26, %46;\n\taddc.cc.u32 %7, %27, %47;\n\taddc.cc.u32 %8, %28, %48;\n\taddc.cc.u32 %9, %29, %49;\n\taddc.cc.u32 %10, %30, %50;\n\taddc.cc.u32 %11, %31, %51;\n\taddc.cc.u32 %12, %32, %52;\n\taddc.cc.u32 %13, %33, %53;\n\taddc.cc.u32 %14, %34, %54;\n\taddc.cc.u32 %15, %35, %55;\n\taddc.cc.u32 %16, %36, %56;\n\taddc.cc.u32 %17, %37, %57;\n\taddc.cc.u32 %18, %38, %58;\n\taddc.u32 %19, %39, %59;"
+        : "=r"(S[0]), "=r"(S[1]), "=r"(S[2]), "=r"(S[3]), "=r"(S[4]), "=r"(S[5]), "=r"(S[6]), "=r"(S[7]), "=r"(S[8]), "=r"(S[9]), "=r"(S[10]), "=r"(S[11]), "=r"(S[12]), "=r"(S[13]), "=r"(S[14]), "=r"(S[15]), "=r"(S[16]), "=r"(S[17]), "=r"(S[18]), "=r"(S[19])
+        : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(A[12]), "r"(A[13]), "r"(A[14]), "r"(A[15]), "r"(A[16]), "r"(A[17]), "r"(A[18]), "r"(A[19]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]), "r"(Bv[12]), "r"(Bv[13]), "r"(Bv[14]), "r"(Bv[15]), "r"(Bv[16]), "r"(Bv[17]), "r"(Bv[18]), "r"(Bv[19]));
+}
+template <>
+__device__ __forceinline__ void add_chain32<22>(uint32_t (&S)[22], const uint32_t (&A)[22], const uint32_t (&Bv)[22]) {
+    asm("add.cc.u32 %0, %22, %44;\n\taddc.cc.u32 %1, %23, %45;\n\taddc.cc.u32 %2, %24, %46;\n\taddc.cc.u32 %3, %25, %47;\n\taddc.cc.u32 %4, %26, %48;\n\taddc.cc.u32 %5, %27, %49;\n\taddc.cc.u32 %6, %28, %50;\n\taddc.cc.u32 %7, %29, %51;\n\taddc.cc.u32 %8, %30, %52;\n\taddc.cc.u32 %9, %31, %53;\n\taddc.cc.u32 %10, %32, %54;\n\taddc.cc.u32 %11, %33, %55;\n\taddc.cc.u32 %12, %34, %56;\n\taddc.cc.u32 %13, %35, %57;\n\taddc.cc.u32 %14, %36, %58;\n\taddc.cc.u32 %15, %37, %59;\n\taddc.cc.u32 %16, %38, %60;\n\taddc.cc.u32 %17, %39, %61;\n\taddc.cc.u32 %18, %40, %62;\n\taddc.cc.u32 %19, %41, %63;\n\taddc.cc.u32 %20, %42, %64;\n\taddc.u32 %21, %43, %65;"
+        : "=r"(S[0]), "=r"(S[1]), "=r"(S[2]), "=r"(S[3]), "=r"(S[4]), "=r"(S[5]), "=r"(S[6]), "=r"(S[7]), "=r"(S[8]), "=r"(S[9]), "=r"(S[10]), "=r"(S[11]), "=r"(S[12]), "=r"(S[13]), "=r"(S[14]), "=r"(S[15]), "=r"(S[16]), "=r"(S[17]), "=r"(S[18]), "=r"(S[19]), "=r"(S[20]), "=r"(S[21])
+        : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(A[4]), "r"(A[5]), "r"(A[6]), "r"(A[7]), "r"(A[8]), "r"(A[9]), "r"(A[10]), "r"(A[11]), "r"(A[12]), "r"(A[13]), "r"(A[14]), "r"(A[15]), "r"(A[16]), "r"(A[17]), "r"(A[18]), "r"(A[19]), "r"(A[20]), "r"(A[21]), "r"(Bv[0]), "r"(Bv[1]), "r"(Bv[2]), "r"(Bv[3]), "r"(Bv[4]), "r"(Bv[5]), "r"(Bv[6]), "r"(Bv[7]), "r"(Bv[8]), "r"(Bv[9]), "r"(Bv[10]), "r"(Bv[11]), "r"(Bv[12]), "r"(Bv[13]), "r"(Bv[14]), "r"(Bv[15]), "r"(Bv[16]), "r"(Bv[17]), "r"(Bv[18]), "r"(Bv[19]), "r"(Bv[20]), "r"(Bv[21]));
 }
 template <>
 __device__ __forceinline__ void add_chain32<24>(uint32_t (&S)[24], const uint32_t (&A)[24], const uint32_t (&Bv)[24]) {

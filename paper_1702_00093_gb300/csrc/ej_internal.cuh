@@ -469,11 +469,14 @@ cudaError_t launch_verify(VerifyConfig c, const uint4 *packed, const uint64_t *p
 // refill).
 // Words per lane the persistent verifier uses for threshold K: its band has at
 // most K + 1 diagonals (the length difference narrows Ukkonen's 2K + 1), one bit
-// each. Every count up to 12 is compiled, then 16 and 24 (K <= 767).
+// each. Every count up to 12 is compiled, then the even ones to 24 (K <= 767): a
+// block of one warp holds windows of W words over as many as 880 / (W + 1) symbols
+// (220 KB of match words), so steps wider than two words would send alphabets near
+// that limit to the G-lane verifier, whose shared memory grows with the string.
 constexpr int PQ_MAX_WORDS = 24;
 inline int pq_words(int32_t K) {
     const int w = (K + 32) / 32;
-    return w <= 12 ? w : w <= 16 ? 16 : w <= PQ_MAX_WORDS ? PQ_MAX_WORDS : w;
+    return w <= 12 || w > PQ_MAX_WORDS ? w : (w + 1) & ~1;
 }
 size_t pq_smem_bytes(int W, uint32_t alpha, int threads);
 int pq_threads_for(int W, uint32_t alpha);   // 0 if no block size fits

@@ -505,7 +505,7 @@ cudaError_t launch_verify_pq(int W, int threads, int spw_force, int wps, const u
         if (B == 8) return launch_pq_tt<WW, 8, 32>(packed, pofs, lens, n, alpha, pairs, np, K, spw_force, wps, vo, s); \
     }
     EJ_PQ(1) EJ_PQ(2) EJ_PQ(3) EJ_PQ(4) EJ_PQ(5) EJ_PQ(6) EJ_PQ(7) EJ_PQ(8) EJ_PQ(9) EJ_PQ(10) EJ_PQ(11) EJ_PQ(12)
-    EJ_PQ(16) EJ_PQ(24)
+    EJ_PQ(14) EJ_PQ(16) EJ_PQ(18) EJ_PQ(20) EJ_PQ(22) EJ_PQ(24)
 #undef EJ_PQ
     return cudaErrorInvalidValue;
 }
