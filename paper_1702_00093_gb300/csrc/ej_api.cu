@@ -772,8 +772,10 @@ uint64_t raw_cap_start(ej_ctx *ctx, int64_t n) {
     return ctx->raw_cap_hint ? ctx->raw_cap_hint : (uint64_t)(n * 4 > 65536 ? n * 4 : 65536);
 }
 
-// Pair slots of the buffers of an attempt with capacity cap: the raw pairs, or
-// the whole tasks of the shared-string verifier.
+// Pair slots of the candidates of an attempt with capacity cap: the pairs, or the
+// tasks of the shared-string verifier that so many distinct pairs can need, whole or
+// not (32 slots each, at most cap + 32 min(n ceil(classes / 2), cap) and a remainder
+// per warp). The list of the pairs handed on and the output hold cap pairs.
 uint64_t back_slots(const Plan &pl, const ej_params *p, const BackState &bs, uint64_t cap) {
     return bs.grouped ? 32 * (uint64_t)group_task_cap(cap, pl.st.n, sx_band(p->K).nclass) : cap;
 }
@@ -781,7 +783,7 @@ uint64_t back_slots(const Plan &pl, const ej_params *p, const BackState &bs, uin
 // The capacity an attempt whose counters are hc would have needed; 0 if it fits.
 uint64_t back_needs(const Plan &pl, const ej_params *p, const BackState &bs, const unsigned long long hc[8], uint64_t cap) {
     if (!bs.grouped) return hc[0] > cap ? hc[0] : 0;
-    return 32 * hc[7] > back_slots(pl, p, bs, cap) ? 32 * hc[7] : 0;
+    return 32 * hc[7] > back_slots(pl, p, bs, cap) || hc[3] > cap ? hc[2] : 0;   // (more than cap distinct pairs)
 }
 
 // verify_after / verify_done (optional): the verifier launch waits for the
@@ -799,9 +801,9 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     while (hsize < 2 * cap) hsize <<= 1;
     const uint64_t slots = back_slots(pl, p, bs, cap);
     uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr;
-    CKS(ensure_t(ctx, B_RAW, (size_t)slots, &raw));
+    CKS(ensure_t(ctx, B_RAW, (size_t)cap, &raw));
     CKS(ensure_t(ctx, B_CAND, (size_t)slots, &cand));
-    CKS(ensure_t(ctx, B_APP, (size_t)slots, &app));
+    CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
     // the verifier and the candidate order it takes
     const bool sx = bs.grouped;
     const int pq_threads = sx ? 0 : pq_choice(ctx, pl, p, bs.vc);
@@ -885,7 +887,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     unsigned int *tickets = nullptr;
     CKS(ensure_t(ctx, B_TICKETS, (size_t)SM_TICKETS, &tickets));
     CK(cudaMemsetAsync(tickets, 0, SM_TICKETS * sizeof(unsigned int), s));
-    VerifyOut vo{nullptr, app, cnt + 3, slots, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
+    VerifyOut vo{nullptr, app, cnt + 3, cap, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
     vo.max_passes = ctx->loop_bound;
     const VerifyConfig &vc = bs.vc;
     if (sx) {
@@ -895,6 +897,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
         const int pq_after = pq_threads_for(pq_words(p->K), p->alphabet_size);
         if (pq_after > 0) {
             vo.defer = raw;
+            vo.defer_cap = cap;
             vo.defer_count = cnt + 8;
         }
         CK(launch_verify_sx(sb.W, pl.packed, pl.pofs, pl.B, pl.lens, n, p->alphabet_size, cand, tasks, cnt + 7,
@@ -905,7 +908,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
             v2.np_dev = cnt + 8;
             CK(launch_verify_pq(pq_words(p->K), pq_after, ctx->sched.slots_per_warp ? ctx->sched.slots_per_warp : 16,
                                 ctx->sched.warps_per_subpartition, pl.packed, pl.pofs, pl.B, pl.lens, n,
-                                p->alphabet_size, raw, (int64_t)slots, p->K, v2, s));
+                                p->alphabet_size, raw, (int64_t)cap, p->K, v2, s));
         }
     } else {
     if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));
@@ -2584,9 +2587,9 @@ int ej_batch_result(ej_batch *b, int32_t i, uint64_t *out, int64_t capacity, int
     if ((uint32_t)hc[6] & DERR_TIMEOUT)
         return fail(ctx, EJ_ERR_TIMEOUT, "the persistent verifier gave up after its bound of loop passes per warp");
     if ((uint32_t)hc[6] & DERR_GUARD) return fail(ctx, EJ_ERR_CUDA, "internal: a work bound was exceeded");
-    if (back_needs(j.pl, &j.p, j.bs, hc, j.cap))
-        return fail(ctx, EJ_ERR_CAPACITY, "raw pairs (%llu) exceed the batch's capacity (%llu): re-create the batch",
-                    hc[0], (unsigned long long)j.cap);
+    if (const uint64_t need = back_needs(j.pl, &j.p, j.bs, hc, j.cap))
+        return fail(ctx, EJ_ERR_CAPACITY, "%s pairs (%llu) exceed the batch's capacity (%llu): re-create the batch",
+                    j.bs.grouped ? "candidate" : "raw", (unsigned long long)need, (unsigned long long)j.cap);
     int64_t cnt = 0;
     int st = EJ_OK;
     if ((int64_t)hc[3] <= small_sort_max()) {

@@ -286,9 +286,11 @@ int group_chunk(int64_t n) { return n >= 65536 ? 16 : n >= 8192 ? 4 : 1; }
 }  // namespace
 
 int64_t group_task_cap(uint64_t cap, int64_t n, uint32_t nclass) {
-    // whole tasks for cap pairs, one partial task per group, and what the warps
-    // reserve and do not use
-    return (int64_t)(cap / 32) + n * (int64_t)nclass + (int64_t)group_blocks(n) * GE_WARPS * group_chunk(n);
+    // whole tasks, the partial ones (the first classes of a string's partial tasks lie
+    // at least two apart, and each holds a pair), and what the warps reserve and do not
+    // use
+    const uint64_t partial = (uint64_t)n * ((nclass + 1) / 2);
+    return (int64_t)(cap / 32 + (partial < cap ? partial : cap)) + (int64_t)group_blocks(n) * GE_WARPS * group_chunk(n);
 }
 
 size_t fingerprint_bytes(int64_t n, int64_t T) { return (size_t)n * ((size_t)(T + 7) / 8) * sizeof(uint4); }

@@ -439,9 +439,10 @@ struct VerifyOut {
     const unsigned long long *unp_dev;
     uint64_t ucap;
     // Shared-string verifier: when set, pairs that outlive the rest of their task
-    // are appended here (room for every pair) and left to a second verifier;
-    // *defer_count (zeroed before the launch) counts them.
+    // are appended here and left to a second verifier; *defer_count (zeroed before the
+    // launch) counts them. Beyond defer_cap pairs it decides them itself.
     uint64_t *defer;
+    uint64_t defer_cap;
     unsigned long long *defer_count;
 };
 
