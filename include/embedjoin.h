@@ -164,6 +164,9 @@ int ej_set_timing(ej_ctx *ctx, int enable);
  * warps_per_block 0 = automatic (at most 4 for lanes_per_pair <= 2). All zero
  * restores the automatic choice. A configuration that cannot cover the band of
  * a later call falls back to the automatic choice. Results never depend on it.
+ * ej_verify takes a tiling that is set here; ej_join takes it in ej_schedule.mode 2,
+ * and in mode 0, where two lanes per pair count for strings of at most 4 symbols
+ * and a mean length below 2048 only (the others take mode 0's verifier).
  */
 int ej_set_verify_config(ej_ctx *ctx, int lanes_per_pair, int words_per_lane, int warps_per_block);
 

@@ -615,6 +615,9 @@ int pick_verify(ej_ctx *ctx, const ej_params *p, const Plan &pl, VerifyConfig *o
     return EJ_OK;
 }
 
+// pick_verify's vc is the tiling that the caller asked for.
+bool tiling_asked(const ej_ctx *ctx, const VerifyConfig &vc) { return ctx->vG > 0 && vc.G == ctx->vG && vc.V == ctx->vV; }
+
 // Verify device pairs; passing pairs (input order) into `out_dev` if it has
 // room (capacity), count in *n_out. If out_dev is null only counts.
 int verify_dev(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *pairs, int64_t np,
@@ -643,7 +646,7 @@ int verify_dev(ej_ctx *ctx, const Plan &pl, const ej_params *p, const uint64_t *
     // fit: its band is half of Ukkonen's and its slots refill (against the grid-
     // strided one: 5000-base reads, K = 150, 0.85 -> 0.26 ms; 900000 text-like
     // candidates, K = 100, 9.7 -> 2.7 ms)
-    const int pq_threads = ctx->vG > 0 ? 0 : pq_threads_for(pq_words(p->K), p->alphabet_size);
+    const int pq_threads = tiling_asked(ctx, vc) ? 0 : pq_threads_for(pq_words(p->K), p->alphabet_size);
     if (pq_threads > 0) {
         CK(cudaMemsetAsync(tickets, 0, SM_TICKETS * sizeof(unsigned int), s));
         CK(launch_verify_pq(pq_words(p->K), pq_threads, 16, 0, pl.packed, pl.pofs, pl.B, pl.lens, pl.st.n,
@@ -722,19 +725,27 @@ bool dense_signatures(const Plan &pl, const ej_params *p) {
     return chance >= 2.0;
 }
 
+// Short strings of at most four symbols take a tiling that the caller asked for in
+// mode 0; the others take mode 0's verifier whatever two-lane tiling is set.
+bool tiling_kept(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
+    return ctx->sched.mode == 0 && p->alphabet_size <= 4 && !long_strings(pl) && tiling_asked(ctx, vc);
+}
+
 // The shared-string verifier: mode 3, or the choice of mode 0; the band within
 // SX_MAX_WORDS words, the warps' rings within the block's budget.
 bool sx_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
     const int W = sx_band(p->K).W;
     if (vc.G != 2 || W > SX_MAX_WORDS || sx_smem_bytes(W, p->alphabet_size) > 220 * 1024) return false;
     if (ctx->sched.mode != 0) return ctx->sched.mode == 3;
+    if (tiling_kept(ctx, pl, p, vc)) return false;
     return p->alphabet_size > 4 ? !long_strings(pl) : dense_signatures(pl, p);
 }
 
 // Threads per block of the persistent verifier this join uses, 0 for none.
 int pq_choice(const ej_ctx *ctx, const Plan &pl, const ej_params *p, const VerifyConfig &vc) {
     const bool want_pq = ctx->sched.mode == 1 ||
-                         (ctx->sched.mode == 0 && (long_strings(pl) || p->alphabet_size <= 4) && !sx_choice(ctx, pl, p, vc));
+                         (ctx->sched.mode == 0 && (long_strings(pl) || p->alphabet_size <= 4) &&
+                          !sx_choice(ctx, pl, p, vc) && !tiling_kept(ctx, pl, p, vc));
     return (vc.G == 2 && want_pq) ? pq_threads_for(pq_words(p->K), p->alphabet_size) : 0;
 }
 
