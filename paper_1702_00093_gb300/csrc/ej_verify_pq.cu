@@ -28,7 +28,7 @@
 // warps is capped (by default one per SM sub-partition), so that a batch larger
 // than the slots keeps every slot busy until the queue runs dry.
 //
-// Early exit. Every other chunk each half computes the minimum value m_h of its
+// Early exit. After every other chunk of a pair each half computes the minimum value m_h of its
 // window (including the top cell). A path of cost <= K crosses both halves'
 // current columns inside their bands, where the values are exact, so
 // m_fwd + m_bwd > K proves ED > K; both lanes of the pair stop.
@@ -267,6 +267,10 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
     int sg = 0;              // the pair's join (merged launch; of the union: the largest K's)
     uint32_t umk = 0;        // union pair: the mask of the joins that list it
     int64_t iters = 0;       // chunks of this warp (bounded by max_iters)
+    // the warp's running pairs have done an odd number of chunks: pairs start together
+    // only where it is even, so that every pair meets the joint bound after its own
+    // second, fourth, ... chunk, whichever pairs ran beside it
+    bool odd = false;
     // a pass of the documented bound is 64 columns, two chunks
     const int64_t max_iters = 2 * (vo.max_passes > 0 ? min(vo.max_passes, (int64_t)1 << 61) : kMaxIters);
     int base = 0;
@@ -288,7 +292,9 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         // time 3.94 ms, four 2.82, eight 2.72; 5.7M DNA pairs, W = 8: 21.6, four 20.5)
         constexpr int REFILL = B == 8 ? 8 : 4;
         const unsigned idle = __ballot_sync(FULL, !have && !exhausted && !rev);
-        const bool refill = idle && (__popc(idle) >= REFILL || !__any_sync(FULL, have));
+        const bool none = !__any_sync(FULL, have);
+        if (none) odd = false;
+        const bool refill = idle && !odd && (none || __popc(idle) >= REFILL);
         while (refill) {
             const bool need = !have && !exhausted;
             const unsigned nb = __ballot_sync(FULL, need && !rev);
@@ -405,11 +411,12 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         }
         T += 32 - __popc(tacc);
         j0 += 32;
-        if ((iters & 1) == 0) {   // the joint bound (every chunk: 2.92 against 2.72 ms on text, W = 4)
+        if (odd) {   // the joint bound (every chunk: 2.92 against 2.72 ms on text, W = 4)
             const int32_t lb = T + diag_min<W>(P, M, s_tab);
             const int32_t lb_other = __shfl_xor_sync(FULL, lb, 1);
             if (have && j0 < ncols && lb + lb_other > kp) rejected = true;
         }
+        odd = !odd;
 
         // finished pairs: all columns run, or rejected (both lanes agree)
         const bool pair_done = have && (rejected || j0 >= ncols);
