@@ -340,9 +340,12 @@ void ej_batch_destroy(ej_batch *batch);
 /*
  * Schedule of ej_join's back half (a performance choice: the output never
  * depends on it; the paper has no counterpart).
- *   mode: 1: persistent verifier where the band fits two lanes per pair (up to
- *     12 words per lane): a fixed grid whose warps pull candidate pairs from a
- *     device work queue and refill a pair slot as soon as its pair is decided;
+ *   mode: 1: persistent verifier where two lanes of the grid-strided one hold
+ *     Ukkonen's band (K <= 351, fewer for large alphabets): a fixed grid whose warps
+ *     pull candidate pairs from a device work queue, a window of up to 24 words of 32
+ *     bits per lane, and refill pair slots as their pairs are decided, several at a
+ *     time (eight, or four with 2-bit codes, and half of the slots where these are
+ *     fewer);
  *     otherwise the grid-strided verifier. 2: always the grid-strided verifier
  *     (one pass over the pairs; a warp's slots start together and the warp ends
  *     with its slowest pair). 3: the shared-string verifier: the candidates are

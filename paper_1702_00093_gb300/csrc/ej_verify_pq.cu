@@ -290,11 +290,13 @@ verify_pq_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
         // W + 1 match words of its pairs however few they are, and pairs that start
         // together mostly end together (956000 text-like pairs, W = 4: one slot at a
         // time 3.94 ms, four 2.82, eight 2.72; 5.7M DNA pairs, W = 8: 21.6, four 20.5)
+        // With fewer slots, half of them.
         constexpr int REFILL = B == 8 ? 8 : 4;
+        const int refill_at = min(REFILL, max(1, (int)spw / 2));
         const unsigned idle = __ballot_sync(FULL, !have && !exhausted && !rev);
         const bool none = !__any_sync(FULL, have);
         if (none) odd = false;
-        const bool refill = idle && !odd && (none || __popc(idle) >= REFILL);
+        const bool refill = idle && !odd && (none || __popc(idle) >= refill_at);
         while (refill) {
             const bool need = !have && !exhausted;
             const unsigned nb = __ballot_sync(FULL, need && !rev);
