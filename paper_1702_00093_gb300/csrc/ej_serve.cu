@@ -144,6 +144,10 @@ struct ej_index {
     // one: concurrent calls never share), at most kPoolSlots of kPoolBytes each
     std::mutex pool_mu;
     std::vector<Slot> pool;
+    // raw pairs of the recent searches, in all and per query (halved with every search
+    // that had fewer; under pool_mu): a search of as many queries starts with room for
+    // them
+    uint64_t raw_recent = 0, raw_per_query = 0;
 };
 
 namespace {
@@ -503,10 +507,17 @@ int ej_index_search(ej_ctx *ctx, ej_index *x, const ej_strings *queries, const i
         qs[(size_t)i] = Query{queries->bytes + a, (int32_t)(b - a), K[i]};   // bytes checked as they are packed
     }
     cudaSetDevice(x->device);
+    const uint64_t nq = (uint64_t)queries->n;
     Slot sl;
+    // this call's capacity: room for some hundred candidates per query, or for those of
+    // the recent searches, before the first retry. It does not follow from the slot's
+    // buffers, which only grow: the call clears a hash set of its capacity.
+    uint64_t cap = std::max<uint64_t>((uint64_t)1 << 16, std::min<uint64_t>(256 * nq, (uint64_t)1 << 22));
     bool pooled = false;
     {
         std::lock_guard<std::mutex> lk(x->pool_mu);
+        const uint64_t raw = std::min(x->raw_recent, x->raw_per_query * nq);
+        cap = std::max<uint64_t>(cap, raw + raw / 4 + 1024);
         if (!x->pool.empty()) {
             sl = x->pool.back();
             x->pool.pop_back();
@@ -514,8 +525,7 @@ int ej_index_search(ej_ctx *ctx, ej_index *x, const ej_strings *queries, const i
         }
     }
     cudaError_t e = pooled ? cudaSuccess : slot_init(sl);
-    // room for some hundred candidates per query before the first retry
-    sl.cap = std::max<uint64_t>(sl.cap, std::min<uint64_t>(256 * (uint64_t)queries->n, (uint64_t)1 << 22));
+    sl.cap = cap;
     std::vector<uint64_t> pairs;
     std::string why;
     CollectStatus cs = COLLECT_RETRY;
@@ -525,8 +535,13 @@ int ej_index_search(ej_ctx *ctx, ej_index *x, const ej_strings *queries, const i
         if (e == cudaSuccess) cs = slot_collect(sl, &pairs, &why);
     }
     {
-        // kept for the next search with its scratch (never after an error)
+        // kept for the next search with its scratch (not after a CUDA error)
         std::lock_guard<std::mutex> lk(x->pool_mu);
+        if (cs == COLLECT_OK) {
+            const uint64_t raw = sl.h_out[0];
+            x->raw_recent = std::max(raw, x->raw_recent / 2);
+            x->raw_per_query = std::max((raw + nq - 1) / nq, x->raw_per_query / 2);
+        }
         if (e == cudaSuccess && sl.device_bytes <= kPoolBytes && x->pool.size() < kPoolSlots) {
             x->pool.push_back(sl);
             sl = Slot{};

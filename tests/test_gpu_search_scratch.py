@@ -1,0 +1,69 @@
+"""Scratch that an index keeps between searches: a search of one query costs the same
+before and after searches that needed room for millions of pairs."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1702_00093_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+DEV = "cuda:0"
+LUT = np.frombuffer(b"ACGT", np.uint8)
+
+
+@pytest.fixture(scope="module")
+def ej():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1702_00093_gb300 import build
+    build.build()
+    from paper_1702_00093_gb300 import embedjoin
+    return embedjoin
+
+
+def _index(ej, ctx, n):
+    """n strings of one prefix and random tails, all in one bucket of the one table:
+    every query of that prefix meets all of them."""
+    rng = np.random.default_rng(n)
+    head = rng.integers(0, 4, size=24)
+    rows = np.concatenate([np.tile(head, (n, 1)), rng.integers(0, 4, size=(n, 24))], axis=1)
+    ss = synth.pack([LUT[r].tobytes() for r in rows], b"ACGT")
+    index = ej.Index(ctx, ej.Strings.from_set(ss, DEV), ej.Params(K=0, r=1, m=1, z=1, L=16, seed=1, alphabet=b"ACGT"))
+
+    def queries(q, seed):
+        t = np.random.default_rng(seed).integers(0, 4, size=(q, 24))
+        return [LUT[np.concatenate([head, r])].tobytes() for r in t]
+
+    return index, queries, ss
+
+
+def _fastest(index, query, K, reps=200):
+    best = 1e9
+    for _ in range(reps):
+        t = time.perf_counter()
+        index.search([query], K)
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+def test_small_search_after_a_large_one(ej):
+    ctx = ej.Context(0)
+    index, queries, ss = _index(ej, ctx, 4000)
+    try:
+        one = LUT[(np.searchsorted(LUT, np.frombuffer(ss.get(0), np.uint8)) + 1) % 4].tobytes()   # meets few or none
+        want = index.search([one], 0)
+        before = _fastest(index, one, 0)
+        for seed in (1, 2):
+            got = index.search(queries(2000, seed) + [ss.get(i) for i in range(4)], 0)   # 8M pairs
+            assert set(got[got >> np.uint64(32) >= 2000].tolist()) >= {((2000 + i) << 32) | i for i in range(4)}
+        for _ in range(8):
+            assert np.array_equal(index.search([one], 0), want)
+        # clearing a hash set for 8M pairs takes about 40 us
+        assert _fastest(index, one, 0) < before + 20e-6
+    finally:
+        index.close()
+        ctx.close()
