@@ -45,18 +45,20 @@ struct DevBuf {
 };
 
 // Grows (never shrinks) a device buffer, at least doubling it, so that growth
-// (whose cudaFree synchronises the device) stays rare; contents are not kept.
-cudaError_t dev_grow(DevBuf &b, size_t bytes, size_t *grown = nullptr) {
+// (whose cudaFree synchronises the device) stays rare; contents are not kept. *held
+// (optional) follows the bytes that the buffer holds.
+cudaError_t dev_grow(DevBuf &b, size_t bytes, size_t *held = nullptr) {
     if (bytes == 0) bytes = 16;
     if (b.p && bytes <= b.bytes) return cudaSuccess;
     if (b.p && bytes < 2 * b.bytes) bytes = 2 * b.bytes;
     if (b.p) cudaFree(b.p);
+    if (held) *held -= b.bytes;
     b.p = nullptr;
     b.bytes = 0;
     const cudaError_t e = cudaMalloc(&b.p, bytes);
     if (e == cudaSuccess) {
         b.bytes = bytes;
-        if (grown) *grown += bytes;
+        if (held) *held += bytes;
     }
     return e;
 }
@@ -104,7 +106,7 @@ struct Slot {
     // the batch
     int64_t Q = 0;
     size_t pre = 0;                        // results copied back with its counters
-    size_t device_bytes = 0;
+    size_t device_bytes = 0;               // held by the buffers
 };
 
 constexpr size_t kOutHead = 16;            // u64 words before the result prefix
@@ -211,25 +213,24 @@ cudaError_t slot_reserve(Slot &sl, const ej_index &x, int64_t Q, int64_t total, 
     }
     const uint64_t cap = sl.cap, hs = hsize_for(cap);
     const int64_t chunk_bound = (total * x.set.B + 127) / 128 + Q + 1;
-    size_t grown = 0;
-    SV(dev_grow(sl.in, in_bytes, &grown));
-    SV(dev_grow(sl.qlens, (size_t)Q * 4, &grown));
-    SV(dev_grow(sl.ccnt, (size_t)(Q + 1) * 4, &grown));
-    SV(dev_grow(sl.qpofs, (size_t)(Q + 2) * 8, &grown));
-    SV(dev_grow(sl.scan, scan_temp_bytes(Q + 1), &grown));
-    SV(dev_grow(sl.qpacked, (size_t)chunk_bound * 16, &grown));
-    SV(dev_grow(sl.qkeys, (size_t)x.T * Q * 8, &grown));
-    SV(dev_grow(sl.raw, cap * 8, &grown));
-    SV(dev_grow(sl.table, hs * 8, &grown));
-    SV(dev_grow(sl.uniq, cap * 8, &grown));
-    SV(dev_grow(sl.bins, (size_t)3 * nc * 8, &grown));
-    SV(dev_grow(sl.cand, cap * 8, &grown));
-    SV(dev_grow(sl.app, cap * 8, &grown));
-    SV(dev_grow(sl.cnt, 8 * 8, &grown));
-    SV(dev_grow(sl.derr, 16, &grown));
-    SV(dev_grow(sl.queue, (size_t)nc * 8, &grown));
-    SV(dev_grow(sl.tickets, (size_t)nc * SM_TICKETS * 4, &grown));
-    sl.device_bytes += grown;
+    size_t *held = &sl.device_bytes;
+    SV(dev_grow(sl.in, in_bytes, held));
+    SV(dev_grow(sl.qlens, (size_t)Q * 4, held));
+    SV(dev_grow(sl.ccnt, (size_t)(Q + 1) * 4, held));
+    SV(dev_grow(sl.qpofs, (size_t)(Q + 2) * 8, held));
+    SV(dev_grow(sl.scan, scan_temp_bytes(Q + 1), held));
+    SV(dev_grow(sl.qpacked, (size_t)chunk_bound * 16, held));
+    SV(dev_grow(sl.qkeys, (size_t)x.T * Q * 8, held));
+    SV(dev_grow(sl.raw, cap * 8, held));
+    SV(dev_grow(sl.table, hs * 8, held));
+    SV(dev_grow(sl.uniq, cap * 8, held));
+    SV(dev_grow(sl.bins, (size_t)3 * nc * 8, held));
+    SV(dev_grow(sl.cand, cap * 8, held));
+    SV(dev_grow(sl.app, cap * 8, held));
+    SV(dev_grow(sl.cnt, 8 * 8, held));
+    SV(dev_grow(sl.derr, 16, held));
+    SV(dev_grow(sl.queue, (size_t)nc * 8, held));
+    SV(dev_grow(sl.tickets, (size_t)nc * SM_TICKETS * 4, held));
     return cudaSuccess;
 }
 

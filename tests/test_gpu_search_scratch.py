@@ -1,5 +1,6 @@
 """Scratch that an index keeps between searches: a search of one query costs the same
-before and after searches that needed room for millions of pairs."""
+before and after searches that needed room for millions of pairs, and scratch that
+grew in steps is kept while what it holds is within the limit."""
 import time
 
 import numpy as np
@@ -64,6 +65,24 @@ def test_small_search_after_a_large_one(ej):
             assert np.array_equal(index.search([one], 0), want)
         # clearing a hash set for 8M pairs takes about 40 us
         assert _fastest(index, one, 0) < before + 20e-6
+    finally:
+        index.close()
+        ctx.close()
+
+
+def test_scratch_that_grew_in_steps_is_kept(ej):
+    """6M, then 8M pairs: buffers of 0.37 GB, then 0.75 GB in place of them (room for 10M
+    pairs in four lists that double, and a hash set of 2^25): less than the limit of
+    1 GiB, which their sum exceeds."""
+    ctx = ej.Context(0)
+    index, queries, _ = _index(ej, ctx, 4000)
+    try:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info(0)[0]
+        index.search(queries(1500, 1), 0)
+        index.search(queries(2000, 2), 0)
+        held = free - torch.cuda.mem_get_info(0)[0]
+        assert 0.6e9 < held < 1.0e9, held
     finally:
         index.close()
         ctx.close()
