@@ -240,7 +240,9 @@ void ej_index_destroy(ej_index *index);
  * hbm_reserve and the server's total stays within hbm_budget (0 = no budget):
  * otherwise it waits while other batches are in flight; with none in flight it
  * is cut to fewer queries, and a single query that still does not fit finishes
- * with status EJ_ERR_OOM. Results are the same as ej_index_search for the same
+ * with status EJ_ERR_OOM. The scratch that ej_index_search keeps with the index is
+ * not the server's and does not count to hbm_budget; where free memory is short it
+ * is given back first. Results are the same as ej_index_search for the same
  * query and K, whatever else is in flight.
  *   ej_server_submit copies the query and returns a request id >= 0, or
  *     -EJ_ERR_INVALID_ARG (byte outside the alphabet, K < 0).

@@ -163,6 +163,17 @@ void index_free(ej_index *x) {
     delete x;
 }
 
+// Gives back the scratch that searches left with the index (false if there is none).
+bool index_trim(ej_index &x) {
+    std::vector<Slot> idle;
+    {
+        std::lock_guard<std::mutex> lk(x.pool_mu);
+        idle.swap(x.pool);
+    }
+    for (Slot &sl : idle) slot_free(sl);
+    return !idle.empty();
+}
+
 struct Query {
     const uint8_t *bytes;
     int32_t len;
@@ -612,7 +623,7 @@ namespace {
 
 void server_loop(ej_server *srv) {
     cudaSetDevice(srv->x->device);
-    const ej_index &x = *srv->x;
+    ej_index &x = *srv->x;
     while (!srv->stop.load()) {
         bool did = false;
         // completions
@@ -691,6 +702,8 @@ void server_loop(ej_server *srv) {
                 fits = growth == 0 || (growth + srv->cfg.hbm_reserve <= free_b &&
                                        (srv->cfg.hbm_budget == 0 ||
                                         srv->device_bytes + growth <= srv->cfg.hbm_budget));
+                // memory that idle searches of this index hold comes first
+                if (!fits && growth + srv->cfg.hbm_reserve > free_b && index_trim(x)) continue;
                 if (fits || others_busy || qs.size() <= 1) break;
                 std::lock_guard<std::mutex> lk(srv->mu);
                 srv->pending.push_front(ss.batch.back());

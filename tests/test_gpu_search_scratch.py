@@ -1,6 +1,7 @@
 """Scratch that an index keeps between searches: a search of one query costs the same
 before and after searches that needed room for millions of pairs, and scratch that
-grew in steps is kept while what it holds is within the limit."""
+grew in steps is kept while what it holds is within the limit, and a server that is
+short of memory gets it back."""
 import time
 
 import numpy as np
@@ -84,5 +85,36 @@ def test_scratch_that_grew_in_steps_is_kept(ej):
         held = free - torch.cuda.mem_get_info(0)[0]
         assert 0.6e9 < held < 1.0e9, held
     finally:
+        index.close()
+        ctx.close()
+
+
+def test_server_takes_the_kept_scratch_back(ej):
+    """A query of 200 MB needs 250 MB; free memory lies 100 MB above the reserve while
+    the index keeps 0.75 GB from a search."""
+    ctx = ej.Context(0)
+    index, queries, ss = _index(ej, ctx, 4000)
+    srv = None
+    try:
+        index.search(queries(2000, 2), 0)
+        torch.cuda.synchronize()
+        srv = ej.Server(index, max_batch=1, inflight=1, max_batch_bytes=1024)
+        srv.close()
+        reserve = torch.cuda.mem_get_info(0)[0] - (100 << 20)
+        srv = ej.Server(index, max_batch=1, inflight=1, max_batch_bytes=1024, hbm_reserve=reserve)
+        long = ss.get(0) + b"ACGT" * (50 << 20)
+        ids = {srv.submit(ss.get(0), 0): [0], srv.submit(long, 0): []}
+        done = {}
+        t = time.time()
+        while len(done) < 2 and time.time() - t < 60:
+            for rid, status, matches, _, _ in srv.poll(wait_us=100000):
+                done[rid] = (status, matches.tolist())
+        assert done == {i: (ej.EJ_OK, m) for i, m in ids.items()}
+        # the index makes new scratch
+        got = index.search([ss.get(5)], 0)
+        assert got.tolist() == [5]
+    finally:
+        if srv:
+            srv.close()
         index.close()
         ctx.close()
