@@ -409,7 +409,7 @@ def run_serving(args, rank, world, local):
                            "parallelism": "single GPU"},
                 "offline_batch": s["offline_batch"], "rates": s["rates"],
                 "identical_to_offline": s["identical_to_offline"], "clocks": s["clocks"]}
-        print(json.dumps(line), flush=True)
+        print_result(line)
 
 
 # ---------------------------------------------------------------------------
@@ -933,6 +933,43 @@ def full_size_join(ej, name, args, rank, dev, stream, flush, world, clk, int_pea
         ctx.close()
 
 
+# The keys of the result line, and of its nested parts where only some are kept. A
+# record of a run keeps the last 3000 characters of its output or so: the line stays
+# well below that, and everything else goes out before it.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches", "e2e", "roofline", "cpu_baseline")
+LINE_PARTS = {"config": ("workload", "n", "Ks", "l2", "parallelism", "autotune"),
+              "clocks": ("sm_mhz", "sm_max_mhz", "reasons", "samples"),
+              "e2e": ("value", "unit", "ms_per_step", "h2d_bytes_per_step", "d2h_bytes_per_step", "error"),
+              "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic"),
+              "cpu_baseline": ("value", "unit", "cores", "kind")}
+
+
+def result_line(full: dict) -> dict:
+    """The keys of LINE_KEYS that `full` has, nested parts cut to LINE_PARTS."""
+    line = {}
+    for k in LINE_KEYS:
+        if k not in full:
+            continue
+        v = full[k]
+        if isinstance(v, dict) and k in LINE_PARTS:
+            v = {q: v[q] for q in LINE_PARTS[k] if q in v}
+            if not v:
+                continue
+        line[k] = v
+    return line
+
+
+def print_result(full: dict):
+    """Whatever the result line cuts or leaves out on lines "detail <key> <JSON>", then
+    the result line: the only line that is a JSON object, and the last one."""
+    line = result_line(full)
+    for k, v in full.items():
+        if line.get(k) != v or k not in line:
+            print(f"detail {k} {json.dumps(v)}")
+    print(json.dumps(line), flush=True)
+
+
 def main():
     args = parse()
     rank, world, local = dist_init()
@@ -1031,7 +1068,7 @@ def main():
             if args.workload == "long_dna" and args.clusters == 2000:
                 got = [p.cpu().numpy().view("uint64") for p in r["result_pairs"]]
                 line["cpu_baseline"]["all_cores"] = cpu_all_cores(ss, params, got)
-        print(json.dumps(line), flush=True)
+        print_result(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
