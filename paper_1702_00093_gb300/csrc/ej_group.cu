@@ -34,13 +34,7 @@ constexpr int GE_WARPS = 8;    // warps per block of the emitting kernel
 constexpr int GE_BLOCKS = 8;   // blocks per SM
 constexpr int GE_KEEP = 160;   // tables whose windows are kept from class to class
 
-__device__ __forceinline__ uint32_t fingerprint(uint64_t k) {
-    k ^= k >> 31;
-    k *= 0x7fb5d329728ea185ull;
-    k ^= k >> 27;
-    k *= 0x81dadef4bc2dd44dull;
-    return (uint32_t)(k >> 48);
-}
+__device__ __forceinline__ uint32_t fingerprint(uint64_t k) { return (uint32_t)(key_hash(k) >> 48); }
 
 // Per record of every sorted table: its string's length beside its id, and for
 // every string its place in the table. counters[1]: the largest run of equal

@@ -20,6 +20,18 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
     return z ^ (z >> 31);
 }
 
+// Hash of a signature: the variant "Mix01" of MurmurHash3's 64-bit finaliser (Stafford
+// 2011). Slots and fingerprints of the bucket kernels, fingerprints of the grouped
+// candidates.
+__device__ __forceinline__ uint64_t key_hash(uint64_t k) {
+    k ^= k >> 31;
+    k *= 0x7fb5d329728ea185ull;
+    k ^= k >> 27;
+    k *= 0x81dadef4bc2dd44dull;
+    k ^= k >> 33;
+    return k;
+}
+
 __host__ __device__ __forceinline__ uint64_t walk_counter(uint32_t l, uint64_t j, uint32_t sigma) {
     return (1ull << 56) | ((uint64_t)l << 48) | (j << 8) | (uint64_t)sigma;
 }

@@ -117,15 +117,6 @@ cudaError_t launch_emit_append(const uint64_t *rec_keys, const uint32_t *rec_ids
 // exactly once, and the length filter ||s_i| - |s_j|| <= K applies per pair.
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ uint64_t key_hash(uint64_t k) {
-    k ^= k >> 31;
-    k *= 0x7fb5d329728ea185ull;
-    k ^= k >> 27;
-    k *= 0x81dadef4bc2dd44dull;
-    k ^= k >> 33;
-    return k;
-}
-
 constexpr uint32_t LIST_END = 0xFFFFFFFFu;
 
 // slot_keys pre-filled with ~0 (never a signature: keys are < 2^64 - 1) and
@@ -523,6 +514,7 @@ cudaError_t launch_bucket_table(const int32_t *lens, int64_t n, int64_t T, const
     return cudaGetLastError();
 }
 
+// MurmurHash3's 64-bit finaliser (Appleby), of a pair.
 __device__ __forceinline__ uint64_t pair_hash(uint64_t k) {
     k ^= k >> 33;
     k *= 0xff51afd7ed558ccdull;
