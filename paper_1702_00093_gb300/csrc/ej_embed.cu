@@ -310,7 +310,7 @@ cudaError_t launch_pack(const uint8_t *bytes, const int64_t *offsets, const int3
                         uint32_t *err, cudaStream_t s) {
     if (n > 0) {
         const int64_t blocks = (n + 7) / 8;   // 8 warps per block
-        const unsigned grid = (unsigned)(blocks > 152 * 16 ? 152 * 16 : blocks);
+        const unsigned grid = (unsigned)(blocks > GRID_SMS * 16 ? GRID_SMS * 16 : blocks);
         if (B == 2)
             pack2_kernel<<<grid, 256, 0, s>>>(bytes, offsets, lens, n, total, code_map, pofs, packed, err);
         else
@@ -1193,7 +1193,7 @@ cudaError_t launch_derive_keys(const uint64_t *src, uint32_t m_src, int64_t n, u
     const int64_t total = (int64_t)r * m * n;
     if (total == 0) return cudaGetLastError();
     const int64_t g = (total + 255) / 256;
-    derive_keys_kernel<<<(unsigned)(g > 152 * 16 ? 152 * 16 : g), 256, 0, s>>>(src, m_src, n, r, m, modulus, dst);
+    derive_keys_kernel<<<(unsigned)(g > GRID_SMS * 16 ? GRID_SMS * 16 : g), 256, 0, s>>>(src, m_src, n, r, m, modulus, dst);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1226,7 +1226,7 @@ cudaError_t launch_keys_modp(uint64_t *keys, int64_t n, uint32_t r, uint32_t m, 
     const int64_t total = (int64_t)r * m * n;
     if (total == 0) return cudaGetLastError();
     const int64_t g = (total + 255) / 256;
-    keys_modp_kernel<<<(unsigned)(g > 152 * 16 ? 152 * 16 : g), 256, 0, s>>>(keys, n, r, m, z, alpha, seed, P);
+    keys_modp_kernel<<<(unsigned)(g > GRID_SMS * 16 ? GRID_SMS * 16 : g), 256, 0, s>>>(keys, n, r, m, z, alpha, seed, P);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1260,7 +1260,7 @@ cudaError_t launch_gather_strings(const uint8_t *bytes, const int64_t *offsets, 
                                   const int64_t *goff, uint8_t *out, cudaStream_t s) {
     if (gn == 0) return cudaGetLastError();
     int64_t g = (gn * 32 + 255) / 256;
-    gather_strings_kernel<<<(unsigned)(g > 152 * 32 ? 152 * 32 : g), 256, 0, s>>>(bytes, offsets, idx, gn, goff, out);
+    gather_strings_kernel<<<(unsigned)(g > GRID_SMS * 32 ? GRID_SMS * 32 : g), 256, 0, s>>>(bytes, offsets, idx, gn, goff, out);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1268,7 +1268,7 @@ cudaError_t launch_gather_strings(const uint8_t *bytes, const int64_t *offsets, 
 cudaError_t launch_remap_pairs(const uint64_t *pairs, int64_t cnt, const int32_t *idx, uint64_t *out, cudaStream_t s) {
     if (cnt == 0) return cudaGetLastError();
     int64_t g = (cnt + 255) / 256;
-    remap_pairs_kernel<<<(unsigned)(g > 152 * 16 ? 152 * 16 : g), 256, 0, s>>>(pairs, cnt, idx, out);
+    remap_pairs_kernel<<<(unsigned)(g > GRID_SMS * 16 ? GRID_SMS * 16 : g), 256, 0, s>>>(pairs, cnt, idx, out);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -10,6 +10,10 @@ namespace ej {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// SMs of a GB300. Grids of kernels that stride over their items are capped at a
+// number of blocks per SM: 8 of 256 threads fill one, 16 or 32 even out the ends.
+constexpr int64_t GRID_SMS = 152;
+
 // SplitMix64 output function (Steele, Lea, Flood 2014): the counter-based
 // source of the random strings R^l (Alg. 1) and of the sampled positions
 // (Thm. 1). Written for the device here; the CPU oracle has its own copy.

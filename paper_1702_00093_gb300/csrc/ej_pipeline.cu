@@ -1097,7 +1097,7 @@ cudaError_t launch_dedup_classes(const uint64_t *raw, uint64_t cap, uint64_t *ta
                                  unsigned long long *counters, cudaStream_t s) {
     if (nc < 1 || nc > 256) return cudaErrorInvalidValue;
     const int64_t g = ((int64_t)cap + 255) / 256;
-    const unsigned gs = (unsigned)(g > 152 * 8 ? 152 * 8 : (g ? g : 1));
+    const unsigned gs = (unsigned)(g > GRID_SMS * 8 ? GRID_SMS * 8 : (g ? g : 1));
     dedup_classes_kernel<<<gs, 256, 0, s>>>(raw, cap, table, hsize, cls, nc, nc == 1 ? cand : uniq, bins, counters);
     note_launches(1);
     if (nc > 1) {
