@@ -2246,6 +2246,7 @@ int ej_join_grouped(ej_ctx *ctx, const ej_strings *S, const ej_params *p, uint64
     sub->vG = ctx->vG;
     sub->vV = ctx->vV;
     sub->vWarps = ctx->vWarps;
+    sub->loop_bound = ctx->loop_bound;
     std::vector<int32_t> idx;
     std::vector<int64_t> goff;
     struct DevBuf {   // the union of the groups' outputs, freed on every return
