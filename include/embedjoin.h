@@ -172,11 +172,14 @@ int ej_set_verify_config(ej_ctx *ctx, int lanes_per_pair, int words_per_lane, in
 
 /*
  * Failure detection (the paper has no counterpart): the persistent verifier
- * (ej_schedule.mode 1, the merged launch of a batch, and the pairs that the
- * shared-string verifier leaves to it) bounds the passes of
- * each warp's work loop, so that a kernel that could not finish its queue
- * stops instead of running on. When the bound runs out the kernel records it
- * and returns, and the call reports EJ_ERR_TIMEOUT; the context stays usable.
+ * bounds the passes of each warp's work loop, so that a kernel that could not
+ * finish its queue stops instead of running on. When the bound runs out the
+ * kernel records it and returns, and the call reports EJ_ERR_TIMEOUT; the context
+ * stays usable. Calls that use it: ej_join and ej_join_grouped in the modes of
+ * ej_schedule that take it, also for the pairs that the shared-string verifier
+ * hands on (so most joins in mode 0), ej_join_plus and ej_verify (unless a tiling
+ * is set), batches (the status comes with ej_batch_result), ej_index_search and
+ * the server, which keep the default bound and report EJ_ERR_CUDA.
  * passes: loop passes per warp (one pass advances the warp's pairs by 64
  * columns); 0 restores the default of 2^24, far above what any valid input
  * needs. A small value is a test hook that makes the bound run out on
@@ -534,7 +537,11 @@ int ej_lsh_candidates(ej_ctx *ctx, const ej_strings *strings, const ej_params *p
  * ED(s_i, s_j) <= params->K (only K and the alphabet of params are used).
  * Pairs need not be sorted or unique; i and j must be < n. Output keeps the
  * input order; `out` must hold n_pairs entries. Exact: the result equals a full
- * Ukkonen band DP. Supports K up to 4095.
+ * Ukkonen band DP. Supports K up to 4095. Runs on the persistent verifier up to
+ * K = 767 where its match words fit (a block of one warp holds windows of W =
+ * ceil((K + 1) / 32) words, even above 12, over 880 / (W + 1) symbols) unless
+ * ej_set_verify_config chose a tiling: EJ_ERR_TIMEOUT if its loop bound runs out
+ * (ej_set_loop_bound).
  */
 int ej_verify(ej_ctx *ctx, const ej_strings *strings, const ej_params *params,
               const uint64_t *pairs, int64_t n_pairs, uint64_t *out, int64_t *n_out, void *stream);
@@ -573,7 +580,8 @@ int ej_verify_noalloc(const ej_strings *strings, const ej_params *params, const 
  * The whole method (Algorithm 3 with Algorithm 2's preprocessing):
  * embed -> sign -> candidates -> verify. Writes up to `capacity` output pairs
  * (sorted ascending); on overflow returns EJ_ERR_CAPACITY with the needed count
- * in *n_out. n < 2 gives 0 pairs. stats may be NULL.
+ * in *n_out. EJ_ERR_TIMEOUT: see ej_set_loop_bound. n < 2 gives 0 pairs. stats
+ * may be NULL.
  */
 int ej_join(ej_ctx *ctx, const ej_strings *strings, const ej_params *params, uint64_t *out,
             int64_t capacity, int64_t *n_out, ej_join_stats *stats, void *stream);
@@ -597,7 +605,7 @@ int ej_join(ej_ctx *ctx, const ej_strings *strings, const ej_params *params, uin
  * match counting and the dedup). Synchronises `stream`.
  * Errors: EJ_ERR_INVALID_ARG (delta <= 0, T < 1, and those of ej_join),
  * EJ_ERR_UNSUPPORTED (n * S * r * m records beyond 2^32), EJ_ERR_CAPACITY
- * (*n_out = needed).
+ * (*n_out = needed), EJ_ERR_TIMEOUT (ej_set_loop_bound).
  */
 int ej_join_plus(ej_ctx *ctx, const ej_strings *strings, const ej_params *params, int32_t delta, int32_t T,
                  uint64_t *out, int64_t capacity, int64_t *n_out, ej_join_stats *stats, void *stream);
