@@ -786,7 +786,7 @@ uint64_t raw_cap_start(ej_ctx *ctx, int64_t n) {
 // Pair slots of the candidates of an attempt with capacity cap: the pairs, or the
 // tasks of the shared-string verifier that so many distinct pairs can need, whole or
 // not (32 slots each, at most cap + 32 min(n ceil(classes / 2), cap) and a remainder
-// per warp). The list of the pairs handed on and the output hold cap pairs.
+// per warp). The output holds cap pairs, the list of those handed on SX_DEFER_MAX a task.
 uint64_t back_slots(const Plan &pl, const ej_params *p, const BackState &bs, uint64_t cap) {
     return bs.grouped ? 32 * (uint64_t)group_task_cap(cap, pl.st.n, sx_band(p->K).nclass) : cap;
 }
@@ -811,8 +811,10 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     uint64_t hsize = 1;
     while (hsize < 2 * cap) hsize <<= 1;
     const uint64_t slots = back_slots(pl, p, bs, cap);
+    // pairs that the shared-string verifier hands on: SX_DEFER_MAX a task at most
+    const uint64_t handed = bs.grouped ? slots / 32 * SX_DEFER_MAX : 0;
     uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr;
-    CKS(ensure_t(ctx, B_RAW, (size_t)cap, &raw));
+    CKS(ensure_t(ctx, B_RAW, (size_t)std::max(cap, handed), &raw));
     CKS(ensure_t(ctx, B_CAND, (size_t)slots, &cand));
     CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
     // the verifier and the candidate order it takes
@@ -908,7 +910,6 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
         const int pq_after = pq_threads_for(pq_words(p->K), p->alphabet_size);
         if (pq_after > 0) {
             vo.defer = raw;
-            vo.defer_cap = cap;
             vo.defer_count = cnt + 8;
         }
         CK(launch_verify_sx(sb.W, pl.packed, pl.pofs, pl.B, pl.lens, n, p->alphabet_size, cand, tasks, cnt + 7,
@@ -919,7 +920,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
             v2.np_dev = cnt + 8;
             CK(launch_verify_pq(pq_words(p->K), pq_after, ctx->sched.slots_per_warp ? ctx->sched.slots_per_warp : 16,
                                 ctx->sched.warps_per_subpartition, pl.packed, pl.pofs, pl.B, pl.lens, n,
-                                p->alphabet_size, raw, (int64_t)cap, p->K, v2, s));
+                                p->alphabet_size, raw, (int64_t)handed, p->K, v2, s));
         }
     } else {
     if (verify_after) CK(cudaStreamWaitEvent(s, verify_after, 0));

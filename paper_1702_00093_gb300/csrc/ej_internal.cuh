@@ -385,6 +385,7 @@ struct SxBand {
     uint32_t width, nclass;
 };
 constexpr int SX_MAX_WORDS = 12;
+constexpr int SX_DEFER_MAX = 8;   // pairs a task hands over at most, once, with its last lanes
 SxBand sx_band(int32_t K);
 size_t sx_smem_bytes(int W, uint32_t alpha);
 int small_sort_max();
@@ -455,10 +456,9 @@ struct VerifyOut {
     const unsigned long long *unp_dev;
     uint64_t ucap;
     // Shared-string verifier: when set, pairs that outlive the rest of their task
-    // are appended here and left to a second verifier; *defer_count (zeroed before the
-    // launch) counts them. Beyond defer_cap pairs it decides them itself.
+    // are appended here (room for SX_DEFER_MAX pairs of every task) and left to a
+    // second verifier; *defer_count (zeroed before the launch) counts them.
     uint64_t *defer;
-    uint64_t defer_cap;
     unsigned long long *defer_count;
 };
 

@@ -46,7 +46,6 @@ namespace {
 
 constexpr int SX_WARPS = 4;       // warps per block
 constexpr int SX_PAIRS = 32;      // slots per task
-constexpr int SX_DEFER_MAX = 8;   // lanes left when a task hands its similar pairs over
 
 // Symbol i (0 <= i < m) of a packed string.
 template <int B>
@@ -290,17 +289,17 @@ verify_sx_kernel(const uint4 *__restrict__ packed, const uint64_t *__restrict__ 
                 } else {
                     const int32_t most = (int32_t)__reduce_max_sync(FULL, running ? (unsigned)(n - j) : 0u);
                     if (vo.defer && __popc(left) <= SX_DEFER_MAX && most > j / 2) {
-                        // similar pairs: to the persistent verifier, unless its list is full
+                        // similar pairs: to the persistent verifier
                         unsigned long long at = 0;
                         if (lane == 0) at = atomicAdd(vo.defer_count, (unsigned long long)__popc(left));
-                        at = __shfl_sync(FULL, at, 0) + __popc(left & ((1u << lane) - 1u));
-                        if (running && at < vo.defer_cap) {
-                            vo.defer[at] = pr;
+                        at = __shfl_sync(FULL, at, 0);
+                        if (running) {
+                            vo.defer[at + __popc(left & ((1u << lane) - 1u))] = pr;
                             deferred = true;
                             running = false;
                             cols_run = j;
                         }
-                        if (!__any_sync(FULL, running)) break;
+                        break;
                     }
                     next_check = j + 64;
                 }

@@ -116,3 +116,34 @@ def test_windows_of_many_tables(ej, r, m):
         assert got[3][:4] == got[2][:4]
         assert got[3][1] == ref.n_candidates > 0
         assert np.array_equal(got[3][4], ref.pairs) and np.array_equal(got[2][4], ref.pairs)
+
+
+def test_handed_on_pairs_do_not_depend_on_the_capacity(ej):
+    """More pairs are handed on than the first capacity has, and fewer than a capacity
+    raised by a larger join before: the same pairs take the second verifier."""
+    rng = np.random.default_rng(6)
+    lut = np.frombuffer(synth.PROTEIN, np.uint8)
+    strs = []
+    for _ in range(80):
+        head, tail = rng.integers(0, 25, size=700), rng.integers(0, 25, size=560)
+        for step in range(8):
+            for k in range(6):
+                end = tail if k < 3 else rng.integers(0, 25, size=560)
+                strs.append(lut[np.concatenate([head, end[:560 - 40 * step]])].tobytes())
+    s = ej.Strings.from_set(synth.pack(strs, synth.PROTEIN), DEV)
+    p = ej.Params(K=300, r=2, m=2, z=12, L=400, seed=1, alphabet=synth.PROTEIN)
+    n = 50000
+    large = ej.Strings(torch.from_numpy(lut[rng.integers(0, 25, size=140 * n)]).to(DEV),
+                       torch.arange(0, 140 * n + 1, 140, dtype=torch.int64, device=DEV))
+    got = []
+    for larger_first in (False, True):
+        ctx = ej.Context(0)
+        ctx.set_schedule(mode=3)
+        if larger_first:
+            ctx.join(large, p, device=DEV)
+        pairs, st = ctx.join(s, p, device=DEV, capacity=1 << 17)
+        got.append((st.n_candidates, st.band_cells, st.verify_word_columns, _u64(pairs)))
+        ctx.close()
+    assert got[0][0] == 80 * 48 * 47 // 2   # above the first capacity of 65536
+    assert got[0][:3] == got[1][:3]
+    assert np.array_equal(got[0][3], got[1][3])
