@@ -706,23 +706,37 @@ constexpr unsigned SMEM_BUCKET_MAX = 256;
 // tables with length windows instead of hashed buckets.
 constexpr unsigned SORTED_BUCKET_MIN = 4096;
 
-// The verifier of mode 0 (measured as whole joins of 20000 strings unless said).
-// More than four symbols: the shared-string verifier for mean lengths below 2048,
-// else the persistent one. At most four symbols (rings of a few hundred bytes per
-// lane): the shared-string verifier when chance alone fills its tasks, i.e. a string
-// meets at least two others that are unrelated, counted as if the z symbols of a
-// signature were uniform (r m n / 2 alphabet^-z; signatures of short strings
-// coincide more often): 1.8M candidates of 100-base reads (5.3) 5.2 (grid-strided)
-// or 5.5 (persistent) -> 1.15 ms, 1500 bases (5.3) 1.9 -> 1.5, 5000 bases at K = 250
-// (85) 26.4 -> 19.5; the persistent one otherwise: 500 bases (1.3) 1.02 against 1.04
-// ms, 5000 reads of 1000 bases (0.3) 0.37 against 0.75, 5000 bases at K = 150 (0)
-// 0.80 against 1.7.
+// The verifier of mode 0. More than four symbols: the shared-string verifier for mean
+// lengths below 2048, else the persistent one. At most four symbols (rings of a few
+// hundred bytes per lane): the shared-string verifier when chance alone fills its
+// tasks (dense_signatures), else the persistent one.
 bool long_strings(const Plan &pl) { return pl.st.n > 0 && pl.st.total / pl.st.n >= 2048; }
 
+// Chance: the unrelated strings before it that a string shares a signature with,
+// counted as if the z symbols of a signature were uniform (r m n / 2 alphabet^-z;
+// signatures of short strings coincide more often). The shared-string verifier cuts a
+// string's candidates into nclass classes and runs a task of few pairs as long as a
+// full one, so the chance it needs grows with the classes and, as the columns to a
+// rejection do, with the words: W nclass / 3, at least 2. Where one block builds each
+// table's buckets (bucket_table_smem), fewer tables than SMs hold the persistent
+// verifier's candidates back, and the line falls with the root of tables / SMs.
+// Placed on 387 joins of 2000 to 60000 reads of 60 to 5000 bases with a chance above 2:
+// the choice takes 2.2% more than the better of the two on average (with 2 as the line
+// for all 7.9%, and no join gets slower by more than 3%). 20000 reads, T tables, whole
+// joins, persistent against shared-string: K = 250, 5000 bases (W nclass = 63), T = 140:
+// 4.3 against 7.6 ms at a chance of 5.3, 9.9 against 9.4 at 21, 25.2 against 18.7 at 85;
+// K = 60, 1500 bases (32), T = 140: 1.8 against 2.2 at 5.3, 3.6 against 2.7 at 21, T = 12:
+// 3.8 against 1.5 at 7.3; K = 6, 100 bases (1), T = 140: 6.7 against 1.2 at 5.3, 3.0 against
+// 1.0 at 1.3, 0.86 each at 0.02 (the floor of 2 leaves these joins slower than they need
+// be; at 5000 to 60000 reads of 250 and more bases the two cross between 0.1 and 5).
 bool dense_signatures(const Plan &pl, const ej_params *p) {
-    double chance = 0.5 * (double)p->r * p->m * (double)pl.st.n;
+    const double tables = (double)p->r * p->m;
+    double chance = 0.5 * tables * (double)pl.st.n;
     for (uint32_t q = 0; q < p->z && chance >= 2.0; q++) chance /= p->alphabet_size;
-    return chance >= 2.0;
+    const SxBand sb = sx_band(p->K);
+    double line = sb.W * (double)sb.nclass / 3.0;
+    if (bucket_table_smem(pl.st.n) > 0 && tables < (double)GRID_SMS) line *= sqrt(tables / (double)GRID_SMS);
+    return chance >= std::max(2.0, line);
 }
 
 // Short strings of at most four symbols take a tiling that the caller asked for in
