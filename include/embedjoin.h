@@ -360,7 +360,8 @@ void ej_batch_destroy(ej_batch *batch);
  *     that outlive the rest of their task are left to the persistent verifier.
  *     0 (default): for alphabets of more than 4 symbols 3 when the strings' mean
  *     length is below 2048, else 1; for the others 3 when a string is expected to
- *     share a signature with at least two others by chance, else 1.
+ *     share a signature with enough others by chance (two, and more where K makes
+ *     the window wide or splits the pairs into many classes), else 1.
  *   chain (batches): how the verifiers of a batch's joins share the GPU: the
  *     persistent ones merged, chained or overlapping, the grid-strided ones
  *     chained unless chain is 1 (the other stages always overlap); see the

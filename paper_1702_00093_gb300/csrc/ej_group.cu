@@ -19,11 +19,11 @@
 //
 // What bounds it: the L2 reads of the fingerprint rows (2 T bytes per string, at
 // most 2 T bytes per raw pair and half of that on average for a new one).
-// 1.06G raw pairs of 200000 protein-like strings (T = 49, K = 40, 622M distinct):
-// 21 ms with the tables' sorting 1.2 ms, where hashed record lists (36 ms), five
-// radix passes over the raw pairs (63 ms) and their compaction (15 ms) took 114 ms;
-// 5003 such strings: 0.19 ms against 3.5 ms for lists in shared memory, one block
-// per table walking buckets of a thousand records.
+// From the signatures to the tasks, 1.06G raw pairs of 200000 protein-like strings
+// (T = 49, K = 40, 622M distinct): 24 ms (the tables' sorting 1.2), where hashed record
+// lists (36 ms), five radix passes over the raw pairs (63 ms) and their compaction
+// (15 ms) took 114 ms; 5003 such strings at K = 60: 0.25 ms against 3.6 ms for lists in
+// shared memory, one block per table walking buckets of a thousand records.
 #include "ej_internal.cuh"
 
 namespace ej {

@@ -28,19 +28,19 @@
 // warps is capped (by default one per SM sub-partition), so that a batch larger
 // than the slots keeps every slot busy until the queue runs dry.
 //
-// Early exit. After every other chunk of a pair each half computes the minimum value m_h of its
-// window (including the top cell). A path of cost <= K crosses both halves'
+// Early exit. After every other chunk of a pair each half computes the minimum value
+// m_h of its window (including the top cell). A path of cost <= K crosses both halves'
 // current columns inside their bands, where the values are exact, so
 // m_fwd + m_bwd > K proves ED > K; both lanes of the pair stop.
 //
-// What bounds it: 32-bit integer instructions, 10 W + about 8 per column. With
-// many pairs (5.4M candidates of 20000 reads of 5000 bases at K = 250) the launch
-// takes 20.5 ms at three warps per sub-partition (23.8 at two, 33.2 at one when
-// slots refilled one by one, 21.7 then at three),
-// against 28.2 ms for the block-aligned window with a test per column that this
-// form replaces; with few (about 13000, K = 250) it is set by the columns of its
-// longest pairs on one warp per sub-partition, 0.38 against 0.50 ms, and 0.25
-// against 0.49 ms at K = 150 (5 words against 8).
+// What bounds it: 32-bit integer instructions, 10 W + about 8 per column. Many pairs
+// fill their pipe: the 5.7M candidates of 20000 reads of 5000 bases at K = 250, z = 7
+// take 20.2 ms at four warps per sub-partition (the choice for so many) or three, 21.5
+// at two and 28.4 at one (that join's default is the shared-string verifier, 17.1 ms);
+// the block-aligned window with a test per column, which this form replaced, took 28.2 ms.
+// Few pairs are set by the columns of the longest on one warp per sub-partition: about
+// 13000 at K = 250 take 0.38 ms (0.50 before), 5200 at K = 150 0.25 ms (0.49 before:
+// 8 words of 64 bits where there are 5 of 32).
 #include <climits>
 
 #include "ej_diag.cuh"

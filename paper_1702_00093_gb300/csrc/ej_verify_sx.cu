@@ -31,12 +31,14 @@
 //
 // What bounds it: 32-bit integer instructions, 10 W + about 8 per column and
 // lane, and 5 per window row and quarter for a minimum.
-// The integer pipe is 79% busy (0.59 instructions issued a cycle, K = 40). 622M
-// candidates of 200000 protein-like strings (K = 40, W = 2): 274 -> 73 ms against two
-// lanes per pair on 64-bit block-aligned words with a minimum every 32 columns
-// (77 ms with the plain minimum, first after 11 K / 8 columns); 30M of 120000
-// text-like strings (K = 200, W = 7): 97.3 -> 39.1 ms and 3.3 ms for the pairs handed
-// over. Narrowing the window as its outer rows drop out was slower (58.6 ms on text):
+// The integer pipe is 79% busy (0.59 instructions issued a cycle, K = 40). With the
+// pairs handed over: 622M candidates of 200000 protein-like strings (K = 40, W = 2) 274 ->
+// 74 ms against two lanes per pair on 64-bit block-aligned words with a minimum every
+// 32 columns (77 ms with the plain minimum, first after 11 K / 8 columns); 30M of 120000
+// text-like strings (K = 200, W = 7) 97.3 -> 40.3 ms. Any test of the list's room in the
+// kernel, even of the whole warp at once, costs protein-like strings 2 to 3%: the list
+// has room for SX_DEFER_MAX pairs of every task.
+// Narrowing the window as its outer rows drop out was slower (58.6 ms on text):
 // the rows that some of 32 pairs still needs leave only in the last third.
 #include "ej_diag.cuh"
 
