@@ -800,15 +800,24 @@ uint64_t raw_cap_start(ej_ctx *ctx, int64_t n) {
 // Pair slots of the candidates of an attempt with capacity cap: the pairs, or the
 // tasks of the shared-string verifier that so many distinct pairs can need, whole or
 // not (32 slots each, at most cap + 32 min(n ceil(classes / 2), cap) and a remainder
-// per warp). The output holds cap pairs, the list of those handed on SX_DEFER_MAX a task.
+// per warp). The list of the pairs handed on has room for SX_DEFER_MAX a task.
 uint64_t back_slots(const Plan &pl, const ej_params *p, const BackState &bs, uint64_t cap) {
     return bs.grouped ? 32 * (uint64_t)group_task_cap(cap, pl.st.n, sx_band(p->K).nclass) : cap;
+}
+
+// Entries of the output of an attempt with capacity cap: no join without tasks has more
+// than cap pairs; with them a string has 32 more (0.3 KB), so that clusters of
+// near-duplicates do not repeat the join.
+uint64_t back_out_cap(const Plan &pl, const ej_params *p, const BackState &bs, uint64_t cap) {
+    return bs.grouped ? std::min(back_slots(pl, p, bs, cap), cap + 32 * (uint64_t)pl.st.n) : cap;
 }
 
 // The capacity an attempt whose counters are hc would have needed; 0 if it fits.
 uint64_t back_needs(const Plan &pl, const ej_params *p, const BackState &bs, const unsigned long long hc[8], uint64_t cap) {
     if (!bs.grouped) return hc[0] > cap ? hc[0] : 0;
-    return 32 * hc[7] > back_slots(pl, p, bs, cap) || hc[3] > cap ? hc[2] : 0;   // (more than cap distinct pairs)
+    return 32 * hc[7] > back_slots(pl, p, bs, cap) || hc[3] > back_out_cap(pl, p, bs, cap)
+               ? hc[2]   // (more than cap distinct pairs)
+               : 0;
 }
 
 // verify_after / verify_done (optional): the verifier launch waits for the
@@ -824,13 +833,13 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     uint32_t *derr = (uint32_t *)ctx->bufs[B_DERR].p;
     uint64_t hsize = 1;
     while (hsize < 2 * cap) hsize <<= 1;
-    const uint64_t slots = back_slots(pl, p, bs, cap);
+    const uint64_t slots = back_slots(pl, p, bs, cap), outs = back_out_cap(pl, p, bs, cap);
     // pairs that the shared-string verifier hands on: SX_DEFER_MAX a task at most
     const uint64_t handed = bs.grouped ? slots / 32 * SX_DEFER_MAX : 0;
     uint64_t *raw = nullptr, *cand = nullptr, *table = nullptr, *app = nullptr;
-    CKS(ensure_t(ctx, B_RAW, (size_t)std::max(cap, handed), &raw));
+    CKS(ensure_t(ctx, B_RAW, (size_t)std::max(outs, handed), &raw));
     CKS(ensure_t(ctx, B_CAND, (size_t)slots, &cand));
-    CKS(ensure_t(ctx, B_APP, (size_t)cap, &app));
+    CKS(ensure_t(ctx, B_APP, (size_t)outs, &app));
     // the verifier and the candidate order it takes
     const bool sx = bs.grouped;
     const int pq_threads = sx ? 0 : pq_choice(ctx, pl, p, bs.vc);
@@ -914,7 +923,7 @@ int back_attempt(ej_ctx *ctx, const Plan &pl, const ej_params *p, const BackStat
     unsigned int *tickets = nullptr;
     CKS(ensure_t(ctx, B_TICKETS, (size_t)SM_TICKETS, &tickets));
     CK(cudaMemsetAsync(tickets, 0, SM_TICKETS * sizeof(unsigned int), s));
-    VerifyOut vo{nullptr, app, cnt + 3, cap, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
+    VerifyOut vo{nullptr, app, cnt + 3, outs, cnt + 2, derr, cnt + 4, cnt + 6, tickets};
     vo.max_passes = ctx->loop_bound;
     const VerifyConfig &vc = bs.vc;
     if (sx) {

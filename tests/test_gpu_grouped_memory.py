@@ -147,3 +147,25 @@ def test_handed_on_pairs_do_not_depend_on_the_capacity(ej):
     assert got[0][0] == 80 * 48 * 47 // 2   # above the first capacity of 65536
     assert got[0][:3] == got[1][:3]
     assert np.array_equal(got[0][3], got[1][3])
+
+
+def test_more_pairs_kept_than_the_first_capacity(ej):
+    """Clusters of 12 equal strings give 5.5 output pairs a string where the first
+    capacity is 4: the first join of a context does no more than the second."""
+    n = 24000
+    rng = np.random.default_rng(8)
+    data = np.frombuffer(synth.PROTEIN, np.uint8)[np.repeat(rng.integers(0, 25, size=(n // 12, 80)), 12, axis=0)]
+    s = ej.Strings(torch.from_numpy(data.reshape(-1).copy()).to(DEV),
+                   torch.arange(0, 80 * n + 1, 80, dtype=torch.int64, device=DEV))
+    p = ej.Params(K=20, r=2, m=2, z=12, L=60, seed=1, alphabet=synth.PROTEIN)
+    want = np.array([(12 * c + i) << 32 | (12 * c + j) for c in range(n // 12) for i in range(12)
+                     for j in range(i + 1, 12)], dtype=np.uint64)
+    ctx = ej.Context(0)
+    ctx.set_schedule(mode=3)
+    launches = []
+    for _ in range(2):
+        pairs, st = ctx.join(s, p, device=DEV, capacity=1 << 18)
+        assert np.array_equal(_u64(pairs), want)
+        launches.append(st.kernel_launches)
+    ctx.close()
+    assert launches[0] == launches[1]
