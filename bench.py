@@ -62,7 +62,7 @@ VERIFY_SOURCE = os.path.join(ROOT, "paper_1702_00093_gb300", "csrc", "ej_verify_
 # one ncu capture of the long-DNA workload: "merged" = the batch's merged launch,
 # "join" = mean over the K=50/150/250 launches of ej_join; valid only while the
 # verify source is the one that was captured
-VERIFY_TRAFFIC = {"source_sha256_prefix": "def08a6506c5d4ca", "bytes_per_launch": {"merged": 13691904, "join": None}}
+VERIFY_TRAFFIC = {"source_sha256_prefix": "982d64ae7c725278", "bytes_per_launch": {"merged": 13640960, "join": None}}
 RECALL_SAMPLES = os.path.join(ROOT, "oracle", "recall_samples.json")
 
 

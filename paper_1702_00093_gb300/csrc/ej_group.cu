@@ -19,7 +19,7 @@
 //
 // What bounds it: the L2 reads of the fingerprint rows (2 T bytes per string, at
 // most 2 T bytes per raw pair and half of that on average for a new one).
-// From the signatures to the tasks, 1.06G raw pairs of 200000 protein-like strings
+// From the signatures to the tasks, 0.80G raw pairs of 200000 protein-like strings
 // (T = 49, K = 40, 622M distinct): 24 ms (the tables' sorting 1.2), where hashed record
 // lists (36 ms), five radix passes over the raw pairs (63 ms) and their compaction
 // (15 ms) took 114 ms; 5003 such strings at K = 60: 0.25 ms against 3.6 ms for lists in
